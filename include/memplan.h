@@ -313,9 +313,10 @@ size_t mp_optimal_workspace_bytes(const mp_batch *batch);
  * opt_peak[b] = the optimum (0 for an empty trace)                int64[B]
  * trace_status[b]: as for mp_plan_greedy_by_size; a trace of more than
  *   MP_OPTIMAL_MAX_TENSORS tensors gets MP_EINVAL.                 int32[B]
- * The search costs n! placements per trace of n tensors.
+ * The search considers n! orders per trace of n tensors and leaves out those
+ * that cannot be the answer.
  * workspace: at least mp_optimal_workspace_bytes(batch) bytes, rules as for
- * mp_plan_greedy_by_size.  Two kernels are enqueued. */
+ * mp_plan_greedy_by_size.  One kernel is enqueued. */
 mp_status mp_plan_optimal(const mp_batch *batch, int64_t *offsets, int64_t *opt_peak, int32_t *trace_status,
                           void *workspace, size_t workspace_bytes, void *stream);
 

@@ -221,8 +221,7 @@ __attribute__((visibility("default"))) mp_status mp_plan_optimal(const mp_batch*
     if (need > 0 && (int64_t)need / (int64_t)sizeof(longlong2) > INT32_MAX) return MP_EINVAL;  // grid too large
     st = check_workspace(need, workspace, workspace_bytes);
     if (st != MP_OK) return st;
-    return from_cuda(mp::launch_optimal(*batch, offsets, opt_peak, trace_status, workspace,
-                                        static_cast<cudaStream_t>(stream)));
+    return from_cuda(mp::launch_optimal(*batch, offsets, opt_peak, trace_status, static_cast<cudaStream_t>(stream)));
 }
 
 __attribute__((visibility("default"))) mp_status mp_slab_layout(const mp_batch* batch, const int64_t* plan_peak,

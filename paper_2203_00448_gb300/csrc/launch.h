@@ -63,7 +63,7 @@ cudaError_t launch_bump(const mp_batch& bt, int64_t* offsets, int64_t* plan_peak
                         cudaStream_t stream);
 
 size_t optimal_workspace_bytes(const mp_batch& bt);
-cudaError_t launch_optimal(const mp_batch& bt, int64_t* offsets, int64_t* opt_peak, int32_t* status, void* workspace,
+cudaError_t launch_optimal(const mp_batch& bt, int64_t* offsets, int64_t* opt_peak, int32_t* status,
                            cudaStream_t stream);
 
 size_t replay_workspace_bytes(const mp_batch& bt);
