@@ -149,7 +149,7 @@ def measured_peaks():
 
 # The sources the fused planner kernel is built from (its traffic in
 # profiles/ncu_traffic.json holds only while these are unchanged).
-PLANNER_SOURCES = ("plan.cu", "common.cuh", "launch.h")
+PLANNER_SOURCES = ("plan.cuh", "phases.cuh", "common.cuh", "launch.h")
 
 
 def kernel_source_digest() -> str:

@@ -16,7 +16,9 @@
 namespace mp {
 
 cudaError_t set_smem_limit(const void* func, size_t bytes) {
-    if (bytes <= 48 * 1024) return cudaSuccess;
+    // without it a kernel may use 48 KB, its static shared memory (up to a few
+    // KB here) included
+    if (bytes <= 32 * 1024) return cudaSuccess;
     static std::mutex mu;
     static std::set<std::pair<int, const void*>> done;
     int dev = 0;
@@ -47,6 +49,24 @@ cudaError_t max_resident_ctas(const void* func, int threads, size_t smem, int* c
         it = cache.emplace(key, std::max(1, sms * per_sm)).first;
     }
     *ctas = it->second;
+    return cudaSuccess;
+}
+
+cudaError_t sm_count(int* sms) {
+    static std::mutex mu;
+    static std::map<int, int> cache;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lock(mu);
+    auto it = cache.find(dev);
+    if (it == cache.end()) {
+        int n = 0;
+        e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) return e;
+        it = cache.emplace(dev, n).first;
+    }
+    *sms = it->second;
     return cudaSuccess;
 }
 

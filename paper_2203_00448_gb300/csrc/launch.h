@@ -17,6 +17,7 @@ constexpr int kBumpThreads = 128;
 constexpr int kOptThreads = 128;
 constexpr int kReplayThreads = 256;
 constexpr int kBreadthThreads = 128;
+constexpr int kBreadthPhaseThreads = 512;  // half of it when the batch has more traces than the GPU SMs
 constexpr int kPlanThreadsSmem = 128;    // one CTA per trace, data in shared memory
 constexpr int kPlanThreadsGlobal = 1024; // one CTA per trace, data in the workspace
 constexpr int kPlanThreadsWide = 512;    // the 64-bit launch: deferred traces, CTA tier included
@@ -35,6 +36,9 @@ cudaError_t set_smem_limit(const void* func, size_t bytes);
 // CTAs of `func` (threads, dynamic shared memory smem) the current device holds
 // at once: SM count x resident CTAs per SM (at least 1); cached per device.
 cudaError_t max_resident_ctas(const void* func, int threads, size_t smem, int* ctas);
+
+// SMs of the current device; cached per device.
+cudaError_t sm_count(int* sms);
 
 // Alignment of every workspace slice.
 constexpr size_t kAlign = 256;
