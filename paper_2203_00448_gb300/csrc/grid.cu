@@ -55,17 +55,21 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "grid.cuh"
+#include "grid_phases.cuh"
 #include "launch.h"
 
 namespace mp {
+
+using namespace grid;
 
 namespace {
 
 constexpr int kGridThreads = 512;             // flow CTA: 16 warps
 constexpr int kGridWarps = kGridThreads / 32;
+static_assert(kGridThreads == kPrepareThreads, "the flow kernel also prepares the traces placed in phases");
 constexpr int kPrepThreads = 512;
 constexpr int kFinishThreads = 256;
-constexpr int32_t kGridLong = 32;             // lives above this many steps: long-lived, placed by a CTA
 // Flow CTA shared memory: a region for the item being placed, then a cache of
 // the batch's long-lived records.  A CTA item uses the region for up to
 // kLongPredPairs predecessor pairs and kLongSuccs successor slots; a warp item
@@ -90,51 +94,6 @@ constexpr long long kGridSpinCycles = MP_TEST_GRID_SPIN_CYCLES;
 #else
 constexpr long long kGridSpinCycles = 1ll << 31;
 #endif
-
-// Queues and counters shared by the whole grid.
-struct GridCtl {
-    int32_t head_s, tail_s;  // warp items: next slot to take, next slot to fill
-    int32_t head_l, tail_l;  // CTA items
-    int32_t total;           // tensors of the traces that passed their checks
-    int32_t placed;          // tensors placed so far
-    int32_t fail;            // a CTA gave up waiting
-    int32_t pad;
-};
-
-// Per-trace state.
-struct TraceInfo {
-    int64_t lo;               // first tensor of the trace in the batch arrays
-    unsigned long long peak;  // largest offset + size
-    unsigned long long key;   // smallest conflicting (min id, max id), packed; ~0 if none
-    int32_t n, T, lw, nlong;  // tensors, steps, longest short life, long-lived tensors
-    int32_t ok;               // 1 once the trace passed its checks
-    int32_t incomplete;       // a tensor was left unplaced
-};
-
-// A tensor in alloc-step order (16 bytes: one vector load).
-struct GRec {
-    int64_t s;
-    int32_t a, f;
-};
-
-struct GridWs {
-    GridCtl* ctl;
-    TraceInfo* ti;
-    int32_t* bend;   // [B][max_steps]: bucket ends by alloc step
-    GRec* rec;       // [B][max_tensors]: alloc-ordered records
-    int32_t* rid;    // tensor id of each record
-    int64_t* off;    // offset of each record (-1 until placed)
-    int32_t* cnt;    // signed predecessor counts
-    int32_t* cls;    // 1: a CTA item (long-lived, or more predecessors than a warp's buffer)
-    int32_t* qs;     // queue of ready warp items (slot ids, -1 = not filled)
-    int32_t* ql;     // queue of ready CTA items
-    int32_t* ll;     // [B][max_tensors]: positions of the long-lived records, ascending
-    int64_t* ovf;    // per long-capable CTA: pairs beyond the shared region
-    int64_t ovf_pairs;
-    int32_t M;       // max_tensors: the slot stride of a trace
-    int32_t TS;      // max_steps: the bucket stride of a trace
-    int64_t hold;    // test hook: the slot that is never queued (-1: none)
-};
 
 struct GridOut {
     int32_t policy;
@@ -303,7 +262,7 @@ __device__ __forceinline__ void push(const GridWs& w, int64_t slot) {
 template <bool kFused>
 __global__ void __launch_bounds__(kPrepThreads) k_grid_prep(mp_batch bt, GridOut out, GridWs w) {
     __shared__ int64_t red[72];
-    __shared__ unsigned long long s_hi, s_lo;
+    __shared__ unsigned long long s_hi, s_lo, s_bits, s_long, s_short;
     __shared__ int s_bad, s_lw, s_nlong;
     const int b = blockIdx.x;
     const int tid = threadIdx.x, nthr = blockDim.x;
@@ -331,7 +290,7 @@ __global__ void __launch_bounds__(kPrepThreads) k_grid_prep(mp_batch bt, GridOut
         if (want_profile) prof[t] = 0;
     }
     if (tid == 0) {
-        s_hi = s_lo = 0;
+        s_hi = s_lo = s_bits = s_long = s_short = 0;
         s_bad = 0;
         s_lw = 1;
         s_nlong = 0;
@@ -341,7 +300,7 @@ __global__ void __launch_bounds__(kPrepThreads) k_grid_prep(mp_batch bt, GridOut
     const int32_t* __restrict__ Fg = bt.free_step + tv.lo;
     const int64_t* __restrict__ Sg = bt.size_bytes + tv.lo;
     bool bad = false;
-    uint64_t sum = 0;
+    uint64_t sum = 0, bits = 0, long_steps = 0, short_steps = 0;
     for (int32_t k = tid; k < n; k += nthr) {
         const int32_t a = __ldg(Ag + k), f = __ldg(Fg + k);
         const int64_t s = __ldg(Sg + k);
@@ -350,6 +309,9 @@ __global__ void __launch_bounds__(kPrepThreads) k_grid_prep(mp_batch bt, GridOut
             continue;
         }
         sum = sat_add(sum, (uint64_t)s);
+        bits |= (uint64_t)s;
+        if (f - a > kGridLong) long_steps += (uint64_t)(f - a);
+        else short_steps += (uint64_t)(f - a);
         atomicAdd(bend + a, 1);
         if (want_profile) {
             atomicAdd(reinterpret_cast<unsigned long long*>(prof + a), (unsigned long long)s);
@@ -358,6 +320,18 @@ __global__ void __launch_bounds__(kPrepThreads) k_grid_prep(mp_batch bt, GridOut
     }
     block_add_size_sum(sum, &s_hi, &s_lo);
     if (bad) s_bad = 1;
+    const unsigned b0 = __reduce_or_sync(0xffffffffu, (unsigned)bits);
+    const unsigned b1 = __reduce_or_sync(0xffffffffu, (unsigned)(bits >> 32));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        long_steps += __shfl_xor_sync(0xffffffffu, long_steps, o);
+        short_steps += __shfl_xor_sync(0xffffffffu, short_steps, o);
+    }
+    if ((tid & 31) == 0) {
+        atomicOr(&s_bits, ((unsigned long long)b1 << 32) | b0);
+        atomicAdd(&s_long, (unsigned long long)long_steps);
+        atomicAdd(&s_short, (unsigned long long)short_steps);
+    }
     __syncthreads();
     if (s_bad || size_sum_overflows(s_hi, s_lo)) {
         fail(s_bad ? MP_EINVAL : MP_EOVERFLOW);
@@ -406,8 +380,16 @@ __global__ void __launch_bounds__(kPrepThreads) k_grid_prep(mp_batch bt, GridOut
         ti->lw = s_lw;
         ti->nlong = nlong;
         ti->incomplete = 0;
+        ti->shift = n > 0 ? __ffsll((long long)s_bits) - 1 : 0;
         ti->ok = 1;
         atomicAdd(&w.ctl->total, n);
+        atomicAdd(&w.ctl->checked, 1);
+        // (a test that holds a tensor back means the dataflow's queues)
+        const bool narrow = (((s_hi << 32) + s_lo) >> ti->shift) <= 0xffffffffull;
+        if (w.p_af != nullptr && w.hold < 0 && narrow) {
+            const int pays = choose_phases(n, nlong, (int64_t)s_long, (int64_t)s_short, T, out.policy);
+            if (pays >= 0) atomicAdd(pays > 0 ? &w.ctl->votes : &w.ctl->neutral, 1);
+        }
     }
 }
 
@@ -1062,7 +1044,36 @@ __device__ int32_t take_slot(const GridWs& w, const int32_t* queue, const int32_
     }
 }
 
-// The persistent grid.  Each CTA first copies the batch's long-lived records
+// Barrier over the grid, whose CTAs are all resident (a cooperative launch):
+// `round` counts its uses from 1.  Every CTA arrives without waiting for
+// anything but this, so it opens as soon as the slowest is there; the wait is
+// bounded like a worker's (false, with the flag raised, when it runs out).
+__device__ __forceinline__ bool grid_barrier(GridCtl* ctl, int32_t round) {
+    __shared__ int32_t s_open;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(&ctl->arrived, 1);
+        const int32_t want = round * (int32_t)gridDim.x;
+        const long long t0 = clock64();
+        int32_t open = 1;
+        while (ld_rlx(&ctl->arrived) < want) {
+            if (ld_rlx(&ctl->fail) || clock64() - t0 > kGridSpinCycles) {
+                atomicExch(&ctl->fail, 1);
+                open = 0;
+                break;
+            }
+            __nanosleep(64);
+        }
+        __threadfence();
+        s_open = open;
+    }
+    __syncthreads();
+    return s_open != 0;
+}
+
+// The persistent grid.  For a batch placed in phases it only prepares what they
+// need (grid_phases.cuh).  Otherwise each CTA first copies the batch's long-lived records
 // into its shared-memory cache (if they fit), then all warps count
 // predecessors; then the first long_ctas CTAs place CTA items (thread 0 takes
 // the next long-queue slot for the whole CTA) and every warp of the others
@@ -1084,6 +1095,11 @@ k_grid_flow(mp_batch bt, int32_t policy, GridWs w, int32_t long_ctas) {
     const int64_t M = w.M;
     const int64_t slots = (int64_t)bt.n_traces * M;
     GridCtl* ctl = w.ctl;
+    if (in_phases(ctl)) {
+        int32_t rounds = 0;
+        far_prepare(bt, w, smem_raw, red, [&]() { return grid_barrier(ctl, ++rounds); });
+        return;
+    }
 
     // the long-lived cache: trace b's records at [s_cbase[b], s_cbase[b + 1])
     LongCache lc;
@@ -1184,6 +1200,17 @@ k_grid_flow(mp_batch bt, int32_t policy, GridWs w, int32_t long_ctas) {
             next = place_short(w, lc, next, policy, buf);
         }
     }
+}
+
+// The traces of a batch chosen for it, placed in phases by a CTA each (a launch of its own:
+// with 1,024 threads instead of the flow kernel's 512 the 20,000-tensor trace
+// takes 12.0 ms instead of 15.7).
+__global__ void __launch_bounds__(kFarThreads, 1) k_grid_phases(mp_batch bt, int32_t policy, GridWs w) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ phases::Shared sh;
+    __shared__ FarShared fs;
+    const TraceInfo* ti = w.ti + blockIdx.x;
+    if (ti->ok && in_phases(w.ctl) && w.ctl->fail == 0) far_place(w, (int32_t)blockIdx.x, policy, smem_raw, sh, fs);
 }
 
 // ---------------------------------------------------------------- finish
@@ -1288,7 +1315,9 @@ __global__ void k_grid_final(mp_batch bt, GridOut out, GridWs w) {
 
 struct GridLayout {
     size_t ctl, ti, bend, rec, rid, off, cnt, cls, qs, ql, ll, ovf, total;
+    size_t p_af, p_sz, p_at, p_cs, p_rk, p_rec, p_win, p_near, p_lr;
     int64_t ovf_pairs;
+    bool phased;
 };
 
 int64_t pow2_ceil(int64_t x) {
@@ -1322,6 +1351,23 @@ GridLayout grid_layout(const mp_batch& bt) {
     // power of two of pairs
     L.ovf_pairs = pow2_ceil((int64_t)M) > kRegionPairs ? pow2_ceil((int64_t)M) : 0;
     L.ovf = take(mul_sat((size_t)kMaxLongCtas, mul_sat((size_t)L.ovf_pairs, 16)));
+    // the arrays of the placement in phases, unless they would take the batch
+    // past the library's own scratch array (mp_plan_greedy_by_size_static)
+    const size_t per_slot = 4 + 4 + 2 + 4 + 4 + sizeof(phases::Rec) + sizeof(phases::Win) + phases::kNear * 2;
+    const size_t more = add_sat(add_sat(mul_sat(slots, per_slot), mul_sat(B, (size_t)kFarMaxLong * 2)), 9 * kAlign);
+    L.phased = bt.max_steps <= 65535 &&
+               (at > MP_PLAN_STATIC_SCRATCH_BYTES || add_sat(at, more) <= MP_PLAN_STATIC_SCRATCH_BYTES);
+    if (L.phased) {
+        L.p_af = take(mul_sat(slots, 4));
+        L.p_sz = take(mul_sat(slots, 4));
+        L.p_at = take(mul_sat(slots, 2));
+        L.p_cs = take(mul_sat(slots, 4));
+        L.p_rk = take(mul_sat(slots, 4));
+        L.p_rec = take(mul_sat(slots, sizeof(phases::Rec)));
+        L.p_win = take(mul_sat(slots, sizeof(phases::Win)));
+        L.p_near = take(mul_sat(slots, phases::kNear * 2));
+        L.p_lr = take(mul_sat(B, (size_t)kFarMaxLong * 2));
+    }
     L.total = at;
     return L;
 }
@@ -1344,6 +1390,18 @@ GridWs grid_ws(const mp_batch& bt, const GridLayout& L, unsigned char* ws) {
     w.M = std::max(bt.max_tensors, 1);
     w.TS = bt.max_steps;
     w.hold = -1;
+    w.p_af = nullptr;
+    if (L.phased) {
+        w.p_af = reinterpret_cast<uint32_t*>(ws + L.p_af);
+        w.p_sz = reinterpret_cast<uint32_t*>(ws + L.p_sz);
+        w.p_at = reinterpret_cast<uint16_t*>(ws + L.p_at);
+        w.p_cs = reinterpret_cast<uint32_t*>(ws + L.p_cs);
+        w.p_rk = reinterpret_cast<uint32_t*>(ws + L.p_rk);
+        w.p_rec = reinterpret_cast<phases::Rec*>(ws + L.p_rec);
+        w.p_win = reinterpret_cast<phases::Win*>(ws + L.p_win);
+        w.p_near = reinterpret_cast<uint16_t*>(ws + L.p_near);
+        w.p_lr = reinterpret_cast<uint16_t*>(ws + L.p_lr);
+    }
     return w;
 }
 
@@ -1361,7 +1419,6 @@ cudaError_t launch_grid_impl(const mp_batch& bt, const GridOut& out, void* works
     k_grid_prep<kFused><<<(unsigned)bt.n_traces, kPrepThreads, 0, stream>>>(bt, out, w);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-
     const void* flow = (const void*)k_grid_flow;
     e = set_smem_limit(flow, kGridSmem);
     if (e != cudaSuccess) return e;
@@ -1378,6 +1435,14 @@ cudaError_t launch_grid_impl(const mp_batch& bt, const GridOut& out, void* works
     void* args[] = {&bt_arg, &policy, &w_arg, &long_ctas};
     e = cudaLaunchCooperativeKernel(flow, dim3((unsigned)grid), dim3(kGridThreads), args, kGridSmem, stream);
     if (e != cudaSuccess) return e;
+
+    if (L.phased && hold < 0) {
+        e = set_smem_limit((const void*)k_grid_phases, kFarSmem);
+        if (e != cudaSuccess) return e;
+        k_grid_phases<<<(unsigned)bt.n_traces, kFarThreads, kFarSmem, stream>>>(bt, policy, w);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
 
     int sms = 0, dev = 0;
     e = cudaGetDevice(&dev);

@@ -1,0 +1,141 @@
+// grid.cuh -- what the planners for batches of a few large traces share: the
+// dataflow over the whole GPU (grid.cu) and the placement in phases by one CTA
+// per trace (grid_phases.cuh).
+#pragma once
+
+#include "common.cuh"
+#include "launch.h"
+#include "phases.cuh"
+
+namespace mp {
+namespace grid {
+
+constexpr int32_t kGridLong = 32;  // lives above this many steps: long-lived
+constexpr int32_t kMaxLongPerThread = 2;
+constexpr int32_t kFarMaxLong = 2048;  // long-lived tensors of a trace placed in phases
+static_assert(kGridLong == phases::kLong, "both planners split lifetimes alike");
+
+// ---- placement in phases by one CTA per trace (grid_phases.cuh)
+constexpr int32_t kFarThreads = 1024;
+constexpr int32_t kPrepareThreads = 512;  // the flow kernel's
+static_assert(kFarMaxLong <= kMaxLongPerThread * kFarThreads, "a thread's share of the long-lived tensors");
+constexpr int32_t kFarMaxTensors = 32767;  // positions and ranks are 16-bit words below phases::kIsLong
+constexpr int32_t kPer = 4;                // buckets of addresses per thread, while a long-lived tensor is placed
+constexpr int32_t kBuckets = kPer * kFarThreads;
+constexpr int32_t kSegments = kBuckets / 8;  // address ranges looked at more closely at a time
+constexpr int32_t kEdges = 1024;           // positions before a window's core whose overlap is kept as bits
+
+// Shared memory of k_far_place for n tensors, nl of them long-lived.
+struct FarLayout {
+    size_t oe, lg_oe, lg_af, heads, edge, mn, mx, flags, seg, total;
+    __host__ __device__ FarLayout(int32_t n, int32_t nl) {
+        auto a16 = [](size_t x) { return (x + 15) & ~size_t(15); };
+        oe = 0;
+        lg_oe = oe + a16((size_t)n * 8);
+        lg_af = lg_oe + a16((size_t)nl * 8);
+        heads = lg_af + a16((size_t)nl * 4);
+        edge = heads + (size_t)phases::kHeads * 2;
+        mn = edge + kEdges / 8;
+        mx = mn + (size_t)kBuckets * 4;
+        flags = mx + (size_t)kBuckets * 4;
+        seg = flags + 2 * kBuckets / 8;
+        total = seg + 2 * (size_t)kSegments * 8;
+    }
+};
+constexpr size_t kFarSmem = 225 * 1024;  // of the 227 KB a CTA may have; the rest is static
+
+// Whether a checked trace can be placed in phases: 1 if one SM is expected to
+// place it sooner than the whole GPU's dataflow, 0 if it can be but matters
+// little (a small trace in a batch of large ones), -1 if not.  Estimates in us.
+// One SM pays for every long-lived tensor with the run before it, more the
+// larger the windows (FIRST: 12 us each with 20,000 tensors, 7 with 2,000; BEST
+// looks at every gap: 43 and 14).  The dataflow pays for its long-lived tensors
+// one after the other where they are live together (`together` of them on
+// average), each the slower the more they are.  Measured, dataflow / phases, ms:
+// long tails of 20,000, 5,000 and 1,500 tensors 25.2 / 12.0, 3.1 / 2.3 and 0.89 /
+// 0.76 (FIRST), 31.4 / 42.9, 3.6 / 4.7 and 1.12 / 1.17 (BEST); seq2seq, 2,000
+// tensors with 40 that span the trace, 1.02 / 0.53 and 1.08 / 0.57.  Without
+// long-lived tensors, or with more neighbours than are listed per short one,
+// the dataflow's width wins.
+__host__ __device__ inline int choose_phases(int64_t n, int64_t nlong, int64_t long_steps, int64_t short_steps,
+                                             int64_t T, int32_t policy) {
+    if (n > kFarMaxTensors || nlong > kFarMaxLong || T > 65535 || 2 * short_steps > (int64_t)phases::kNear * T)
+        return -1;
+    if (FarLayout((int32_t)n, (int32_t)nlong).total > kFarSmem) return -1;
+    if (n <= 1024) return 0;
+    if (nlong == 0) return -1;
+    const int64_t together = long_steps / T;
+    const int64_t phased = 150 + nlong * (policy == MP_FIT_FIRST ? 6 + n / 3300 : 10 + n / 600);
+    const int64_t flow = 45 * together + 3 * together * together / 10;
+    return phased <= flow ? 1 : -1;
+}
+
+// Queues and counters shared by the whole grid.
+struct GridCtl {
+    int32_t head_s, tail_s;  // warp items: next slot to take, next slot to fill
+    int32_t head_l, tail_l;  // CTA items
+    int32_t total;           // tensors of the traces that passed their checks
+    int32_t placed;          // tensors placed so far
+    int32_t fail;            // a CTA gave up waiting
+    int32_t checked;         // traces that passed their checks ...
+    int32_t votes, neutral;  // ... for which phases pay, and which fit them (choose_phases)
+    int32_t arrived;         // CTAs that reached the grid's barriers, all told
+    int32_t pad;
+};
+
+// Whether the batch's traces are placed by one CTA each in phases
+// (grid_phases.cuh) instead of by the dataflow: all of them or none, since the
+// two would run one after the other (once k_grid_prep has finished).
+__device__ __forceinline__ bool in_phases(const GridCtl* ctl) {
+    return ctl->votes > 0 && ctl->votes + ctl->neutral == ctl->checked;
+}
+
+// Per-trace state.
+struct TraceInfo {
+    int64_t lo;               // first tensor of the trace in the batch arrays
+    unsigned long long peak;  // largest offset + size
+    unsigned long long key;   // smallest conflicting (min id, max id), packed; ~0 if none
+    int32_t n, T, lw, nlong;  // tensors, steps, longest short life, long-lived tensors
+    int32_t ok;               // 1 once the trace passed its checks
+    int32_t incomplete;       // a tensor was left unplaced
+    int32_t shift;            // every size is a multiple of 1 << shift (a unit)
+};
+
+// A tensor in alloc-step order (16 bytes: one vector load).
+struct GRec {
+    int64_t s;
+    int32_t a, f;
+};
+
+struct GridWs {
+    GridCtl* ctl;
+    TraceInfo* ti;
+    int32_t* bend;   // [B][max_steps]: bucket ends by alloc step
+    GRec* rec;       // [B][max_tensors]: alloc-ordered records
+    int32_t* rid;    // tensor id of each record
+    int64_t* off;    // offset of each record (-1 until placed)
+    int32_t* cnt;    // signed predecessor counts
+    int32_t* cls;    // 1: a CTA item (long-lived, or more predecessors than a warp's buffer)
+    int32_t* qs;     // queue of ready warp items (slot ids, -1 = not filled)
+    int32_t* ql;     // queue of ready CTA items
+    int32_t* ll;     // [B][max_tensors]: positions of the long-lived records, ascending
+    int64_t* ovf;    // per long-capable CTA: pairs beyond the shared region
+    int64_t ovf_pairs;
+    int32_t M;       // max_tensors: the slot stride of a trace
+    int32_t TS;      // max_steps: the bucket stride of a trace
+    int64_t hold;    // test hook: the slot that is never queued (-1: none)
+    // For traces placed in phases, by slot (stable: alloc step, then id), or
+    // by rank: null if no trace of the batch can be.
+    uint32_t* p_af;  // lifetime: alloc | free << 16
+    uint32_t* p_sz;  // size in units
+    uint16_t* p_at;  // the record's position in rec / off
+    uint32_t* p_cs;  // 1 + first position of its component of short lifetimes (0: long-lived)
+    uint32_t* p_rk;  // priority rank
+    phases::Rec* p_rec;    // by rank
+    phases::Win* p_win;    // by rank
+    uint16_t* p_near;      // by rank: phases::kNear positions
+    uint16_t* p_lr;        // [B][kFarMaxLong]: ranks of the long-lived tensors, ascending
+};
+
+}  // namespace grid
+}  // namespace mp

@@ -85,8 +85,9 @@ cudaError_t launch_peak(const mp_batch& bt, const int64_t* offsets, int64_t* pla
                         cudaStream_t stream);
 
 // Batches of at most kGridMaxTraces traces whose max_tensors exceeds
-// kGridMinTensors -- a few large traces -- are planned by the grid-wide
-// dataflow (grid.cu); every other batch by one CTA per trace (plan.cu).
+// kGridMinTensors -- a few large traces -- are planned by the
+// grid-wide planners (grid.cu, grid_phases.cu); every other batch by one CTA
+// per trace (plan.cuh).
 constexpr int32_t kGridMinTensors = 1024;
 constexpr int32_t kGridMaxTraces = 32;
 bool grid_path(const mp_batch& bt);

@@ -42,9 +42,12 @@ namespace phases {
 constexpr int32_t kLong = 32;          // lives above this many steps are long
 constexpr int32_t kMaxLong = 768;      // long tensors a trace may have here
 constexpr int32_t kMaxTensors = 4096;  // tensors a trace may have here
+constexpr uint32_t kLongestChain = 1024;  // positions a chain may span beside long tensors: one warp walks it, the
+                                       // general paths' queues place its members side by side
 constexpr int32_t kBatch = 512;        // tensors inserted into the sorted list at a time
 constexpr int32_t kHeads = 1024;       // chains of a run listed at a time
 constexpr int32_t kChunk = 16;         // sorted-list entries per thread: kMaxTensors / the fewest threads
+constexpr int32_t kNear = 32;          // neighbours listed per short tensor of a large trace (grid_phases.cu)
 constexpr int32_t kThreadChain = 8;    // chains up to this long within a run can be walked by one thread
 constexpr int32_t kListRun = 64;       // runs from this length on list the gaps between the long tensors first
 constexpr int32_t kFewPending = 8;     // up to this many are inserted by comparison with every entry
@@ -59,7 +62,7 @@ struct __align__(16) Rec {
     uint16_t a, f;        // lifetime [a, f)
     uint16_t pos;         // alloc-order position
     uint16_t next, prev;  // ranks of the neighbours in its chain (component of short lifetimes)
-    uint16_t pad;
+    uint16_t many;        // kFar: more than kNear neighbours, not listed
 };
 // Alloc-order positions of the short tensors that can overlap it: [w0, w1);
 // those from `core` on are allocated during its life.
@@ -243,7 +246,10 @@ __device__ void block_sort(uint64_t (&k)[E], uint64_t* buf) {
     __syncthreads();
 }
 
-// The trace being placed.
+// The trace being placed.  kFar: a large trace whose records by rank and
+// lifetimes are in global memory, with the neighbours of its short tensors
+// listed beforehand (grid_phases.cu).
+template <bool kFar>
 struct Ctx {
     uint2* oe;            // by position: (offset, end) in units; (0, 0) until placed
     const uint32_t* af;   // by position: alloc step | free step << 16
@@ -255,6 +261,7 @@ struct Ctx {
     const uint32_t* mask; // by rank
     uint64_t* pk;         // kBatch keys of tensors being inserted; gaps (start << 32 | length) otherwise
     uint16_t* heads;      // kHeads ranks
+    const uint16_t* near; // kFar, by rank: positions of the kNear short tensors it overlaps (kNone: no more)
     int32_t policy;
 };
 
@@ -320,7 +327,7 @@ struct Near {
 
 // Places the short tensor of rank r, whose gaps between long ones are listed
 // and whose window has a mask, with one thread; returns its end.
-__device__ __forceinline__ uint32_t place_short_alone(const Ctx& c, int32_t r, const Longs& lg) {
+__device__ __forceinline__ uint32_t place_short_alone(const Ctx<false>& c, int32_t r, const Longs& lg) {
     const Rec rc = c.rec[r];
     const Near nr = {c.oe + c.win[r].w0, c.mask[r], rc.s};
     const uint32_t s = rc.s;
@@ -350,7 +357,7 @@ __device__ __forceinline__ uint32_t place_short_alone(const Ctx& c, int32_t r, c
 }
 
 // The same with one warp, a gap per lane.
-__device__ __forceinline__ uint32_t place_short_listed(const Ctx& c, int32_t r, const Longs& lg) {
+__device__ __forceinline__ uint32_t place_short_listed(const Ctx<false>& c, int32_t r, const Longs& lg) {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const Rec rc = c.rec[r];
@@ -395,7 +402,8 @@ __device__ __forceinline__ uint32_t place_short_listed(const Ctx& c, int32_t r, 
 }
 
 // Places the short tensor of rank r with one warp; returns its end.
-__device__ __forceinline__ uint32_t place_short(const Ctx& c, int32_t r, const Longs& lg) {
+template <bool kFar>
+__device__ __forceinline__ uint32_t place_short(const Ctx<kFar>& c, int32_t r, const Longs& lg) {
     const unsigned full = 0xffffffffu;
     const int32_t nlp = lg.nlp;
     const int lane = threadIdx.x & 31;
@@ -409,14 +417,21 @@ __device__ __forceinline__ uint32_t place_short(const Ctx& c, int32_t r, const L
         return v;
     };
     uint2 p0 = make_uint2(0, 0), p1 = make_uint2(0, 0);
-    if (w0 + lane < w1) p0 = load(w0 + lane);
-    if (w0 + 32 + lane < w1) p1 = load(w0 + 32 + lane);
-    const bool wide = w1 - w0 > 64;
+    int32_t rest = w0 + 64;  // window positions from here on are not held in p0, p1
+    if constexpr (kFar) {
+        const uint32_t q = c.near[(size_t)r * kNear + lane];  // (loaded with the record, whatever it says)
+        if (!rc.many && q != kNone) p0 = c.oe[q];
+        rest = rc.many ? w0 : w1;
+    } else {
+        if (w0 + lane < w1) p0 = load(w0 + lane);
+        if (w0 + 32 + lane < w1) p1 = load(w0 + 32 + lane);
+    }
+    const bool wide = rest < w1;
     auto each = [&](auto&& fn) {
         fn(p0.x, p0.y);
-        fn(p1.x, p1.y);
+        if (!kFar) fn(p1.x, p1.y);
         if (wide)
-            for (int32_t q = w0 + 64 + lane; q < w1; q += 32) {
+            for (int32_t q = rest + lane; q < w1; q += 32) {
                 const uint2 v = load(q);
                 fn(v.x, v.y);
             }
@@ -466,6 +481,8 @@ __device__ __forceinline__ uint32_t place_short(const Ctx& c, int32_t r, const L
     const bool first = c.policy == MP_FIT_FIRST;
     uint32_t carry = 0;  // largest end of the long obstacles so far
     bool found = false;
+    uint32_t lane_best = 0, lane_len = 0xffffffffu;  // BEST: the best untouched gap this lane saw
+    const unsigned near0 = __ballot_sync(full, p0.y != 0), near1 = __ballot_sync(full, p1.y != 0);
     for (int32_t k0 = 0; k0 < nlp && !found; k0 += 32) {
         const int32_t k = k0 + lane;
         bool hit = false;
@@ -476,10 +493,40 @@ __device__ __forceinline__ uint32_t place_short(const Ctx& c, int32_t r, const L
             if (hit) v = c.lg_oe[k];
         }
         if (!__any_sync(full, hit)) continue;
-        const uint32_t incl = warp_incl_max(v.y);
-        uint32_t prev = __shfl_up_sync(full, incl, 1);
-        prev = lane == 0 ? carry : umax2(prev, carry);
-        unsigned g = __ballot_sync(full, hit && v.x >= prev && v.x - prev >= s);
+        // the largest end before each: that of the obstacle before it, as they
+        // lie side by side unless two that never meet overlap in address
+        const unsigned hm = __ballot_sync(full, hit), before = hm & ((1u << lane) - 1u);
+        uint32_t prev = __shfl_sync(full, v.y, before ? 31 - __clz(before) : 0);
+        prev = before ? umax2(prev, carry) : carry;
+        if (__any_sync(full, hit && v.y < prev)) {
+            const uint32_t incl = warp_incl_max(v.y);
+            prev = __shfl_up_sync(full, incl, 1);
+            prev = lane == 0 ? carry : umax2(prev, carry);
+        }
+        bool fits = hit && v.x >= prev && v.x - prev >= s;
+        if (!first && !wide) {
+            // most gaps meet no window tensor: those are compared as they
+            // are, a lane each (looking into every one took a warp reduction
+            // or two per gap; the 20,000-tensor trace, BEST: @FARBEST@)
+            bool touched = false;
+            for (unsigned b = near0; b; b &= b - 1) {
+                const int src = __ffs(b) - 1;
+                touched |= (__shfl_sync(full, p0.x, src) < v.x) & (__shfl_sync(full, p0.y, src) > prev);
+            }
+            if (!kFar)
+                for (unsigned b = near1; b; b &= b - 1) {
+                    const int src = __ffs(b) - 1;
+                    touched |= (__shfl_sync(full, p1.x, src) < v.x) & (__shfl_sync(full, p1.y, src) > prev);
+                }
+            if (fits && !touched) {
+                if (v.x - prev < lane_len) {
+                    lane_len = v.x - prev;
+                    lane_best = prev;
+                }
+                fits = false;
+            }
+        }
+        unsigned g = __ballot_sync(full, fits);
         while (g) {  // gaps between long obstacles that hold the tensor, ascending
             const int src = __ffs(g) - 1;
             g &= g - 1;
@@ -494,7 +541,7 @@ __device__ __forceinline__ uint32_t place_short(const Ctx& c, int32_t r, const L
                 holes(g0, g1);
             }
         }
-        carry = umax2(carry, __shfl_sync(full, incl, 31));
+        carry = umax2(carry, __reduce_max_sync(full, v.y));
     }
     if (!found) {
         if (first) {
@@ -504,6 +551,12 @@ __device__ __forceinline__ uint32_t place_short(const Ctx& c, int32_t r, const L
             each([&](uint32_t, uint32_t pe) { top = umax2(top, pe); });
             top = umax2(__reduce_max_sync(full, top), carry);
             holes(carry, top);
+            const uint32_t ln = __reduce_min_sync(full, lane_len);
+            const uint32_t at = __reduce_min_sync(full, lane_len == ln ? lane_best : 0xffffffffu);
+            if (ln < best_len || (ln == best_len && at < best)) {  // (both none: best is overwritten below)
+                best_len = ln;
+                best = at;
+            }
             if (best_len == 0xffffffffu) best = top;
         }
     }
@@ -516,7 +569,7 @@ __device__ __forceinline__ uint32_t place_short(const Ctx& c, int32_t r, const L
 // per lane, when no gap between long tensors needs a look: everything goes
 // above lg.top.  The next member's entries (which depend on no offset) are
 // loaded while the current one is placed.
-__device__ __forceinline__ uint32_t walk_plain(const Ctx& c, int32_t r, int32_t r1, const Longs& lg) {
+__device__ __forceinline__ uint32_t walk_plain(const Ctx<false>& c, int32_t r, int32_t r1, const Longs& lg) {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const bool first = c.policy == MP_FIT_FIRST;
@@ -581,7 +634,8 @@ __device__ __forceinline__ uint32_t walk_plain(const Ctx& c, int32_t r, int32_t 
 // span the trace, 16 warps: 164 K cycles by warps alone, 78 K with threads: a
 // thread's walk costs about 20 times fewer issue slots.)  The caller puts a barrier after it.  Returns the largest
 // end this thread or its warp placed.
-__device__ __forceinline__ uint32_t run_chains(const Ctx& c, int32_t r0, int32_t r1, const Longs& lg, Shared& sh) {
+template <bool kFar>
+__device__ __forceinline__ uint32_t run_chains(const Ctx<kFar>& c, int32_t r0, int32_t r1, const Longs& lg, Shared& sh) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     uint32_t mx = 0;
     auto is_head = [&](int32_t r) {
@@ -589,13 +643,19 @@ __device__ __forceinline__ uint32_t run_chains(const Ctx& c, int32_t r0, int32_t
         return p == kNone || p < r0;
     };
     auto warp_walk = [&](int32_t r) {
-        if (lg.ng == 0) {  // no long tensors' gaps to look at
-            mx = umax2(mx, walk_plain(c, r, r1, lg));
-            return;
+        if constexpr (!kFar) {
+            if (lg.ng == 0) {  // no long tensors' gaps to look at
+                mx = umax2(mx, walk_plain(c, r, r1, lg));
+                return;
+            }
         }
         while (r < r1) {  // (kNone is past every rank)
-            const bool masked = lg.ng >= 0 && !c.win[r].wide;
-            mx = umax2(mx, masked ? place_short_listed(c, r, lg) : place_short(c, r, lg));
+            bool listed = false;
+            if constexpr (!kFar) {
+                listed = lg.ng >= 0 && !c.win[r].wide;
+                if (listed) mx = umax2(mx, place_short_listed(c, r, lg));
+            }
+            if (!listed) mx = umax2(mx, place_short(c, r, lg));
             r = c.rec[r].next;
         }
     };
@@ -632,9 +692,11 @@ __device__ __forceinline__ uint32_t run_chains(const Ctx& c, int32_t r0, int32_t
                 i = __shfl_sync(0xffffffffu, i, 0);
                 if (i >= (alone ? nh1 : nh)) break;
                 if (alone) {
-                    if (i + lane < nh1)
-                        for (int32_t r = c.heads[kHeads - 1 - i - lane]; r < r1; r = c.rec[r].next)
-                            mx = umax2(mx, place_short_alone(c, r, lg));
+                    if constexpr (!kFar) {
+                        if (i + lane < nh1)
+                            for (int32_t r = c.heads[kHeads - 1 - i - lane]; r < r1; r = c.rec[r].next)
+                                mx = umax2(mx, place_short_alone(c, r, lg));
+                    }
                     __syncwarp();
                 } else {
                     warp_walk(c.heads[i]);
@@ -648,7 +710,7 @@ __device__ __forceinline__ uint32_t run_chains(const Ctx& c, int32_t r0, int32_t
 // Inserts m placed tensors, pend(i) being the position of the i-th, into the
 // sorted list of len entries; ends with a barrier.
 template <typename Pend>
-__device__ __forceinline__ void insert_pending(const Ctx& c, int32_t len, int32_t m, Pend&& pend, Shared& sh) {
+__device__ __forceinline__ void insert_pending(const Ctx<false>& c, int32_t len, int32_t m, Pend&& pend, Shared& sh) {
     const int32_t t = (int32_t)threadIdx.x, nt = (int32_t)blockDim.x;
     for (int32_t done = 0; done < m; done += kBatch) {
         const int32_t mb = min(kBatch, m - done);
@@ -772,10 +834,54 @@ __device__ __forceinline__ void insert_pending(const Ctx& c, int32_t len, int32_
     }
 }
 
+// Adds the long tensor x, placed at o, to the nlp placed long ones (at most
+// kPer per thread), whose entries above it move up by one; ends with a barrier.
+template <int kPer, bool kFar>
+__device__ __forceinline__ void add_long(const Ctx<kFar>& c, const Rec& rc, uint32_t o, int32_t nlp) {
+    const int32_t t = (int32_t)threadIdx.x, nt = (int32_t)blockDim.x;
+    const uint32_t s = rc.s;
+    uint2 v[kPer];
+    uint32_t af[kPer];
+#pragma unroll
+    for (int x = 0; x < kPer; ++x) {
+        const int32_t k = t + x * nt;
+        if (k < nlp) {
+            v[x] = c.lg_oe[k];
+            af[x] = c.lg_af[k];
+        }
+    }
+    // its own place: after the last entry at or below it
+    bool mine = t == 0 && (nlp == 0 || v[0].x > o);
+    int32_t here = 0;
+#pragma unroll
+    for (int x = 0; x < kPer; ++x) {
+        const int32_t k = t + x * nt;
+        if (k < nlp && v[x].x <= o && (k + 1 == nlp || c.lg_oe[k + 1].x > o)) {
+            mine = true;
+            here = k + 1;
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int x = 0; x < kPer; ++x) {
+        const int32_t k = t + x * nt;
+        if (k < nlp && v[x].x > o) {
+            c.lg_oe[k + 1] = v[x];
+            c.lg_af[k + 1] = af[x];
+        }
+    }
+    if (mine) {
+        c.lg_oe[here] = make_uint2(o, o + s);
+        c.lg_af[here] = (uint32_t)rc.a | ((uint32_t)rc.f << 16);
+    }
+    if (t == 0) c.oe[rc.pos] = make_uint2(o, o + s);
+    __syncthreads();
+}
+
 // Places the long tensor of rank r with the whole CTA over the sorted list of
 // len placed tensors, and adds it to the nlp placed long ones; ends with a
 // barrier.  Returns its end.
-__device__ __forceinline__ uint32_t place_long(const Ctx& c, int32_t r, int32_t len, int32_t nlp, Shared& sh) {
+__device__ __forceinline__ uint32_t place_long(const Ctx<false>& c, int32_t r, int32_t len, int32_t nlp, Shared& sh) {
     const int32_t t = (int32_t)threadIdx.x, nt = (int32_t)blockDim.x;
     const unsigned full = 0xffffffffu;
     const Rec rc = c.rec[r];
@@ -826,51 +932,14 @@ __device__ __forceinline__ uint32_t place_long(const Ctx& c, int32_t r, int32_t 
     uint32_t o;
     if (first) o = sh.best32 != 0xffffffffu ? sh.best32 : top;
     else o = sh.best != ~0ull ? (uint32_t)sh.best : top;
-    // into the list of placed long tensors: the entries above it move up by one
-    constexpr int kPer = (kMaxLong + 255) / 256;
-    uint2 v[kPer];
-    uint32_t af[kPer];
-#pragma unroll
-    for (int x = 0; x < kPer; ++x) {
-        const int32_t k = t + x * nt;
-        if (k < nlp) {
-            v[x] = c.lg_oe[k];
-            af[x] = c.lg_af[k];
-        }
-    }
-    // its own place: after the last entry at or below it
-    bool mine = t == 0 && (nlp == 0 || v[0].x > o);
-    int32_t here = 0;
-#pragma unroll
-    for (int x = 0; x < kPer; ++x) {
-        const int32_t k = t + x * nt;
-        if (k < nlp && v[x].x <= o && (k + 1 == nlp || c.lg_oe[k + 1].x > o)) {
-            mine = true;
-            here = k + 1;
-        }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int x = 0; x < kPer; ++x) {
-        const int32_t k = t + x * nt;
-        if (k < nlp && v[x].x > o) {
-            c.lg_oe[k + 1] = v[x];
-            c.lg_af[k + 1] = af[x];
-        }
-    }
-    if (mine) {
-        c.lg_oe[here] = make_uint2(o, o + s);
-        c.lg_af[here] = (uint32_t)rc.a | ((uint32_t)rc.f << 16);
-    }
-    if (t == 0) c.oe[rc.pos] = make_uint2(o, o + s);
-    __syncthreads();
+    add_long<(kMaxLong + 255) / 256>(c, rc, o, nlp);
     return o + s;
 }
 
 // Lists the gaps between the placed long tensors that hold the smallest tensor
 // of the run [r0, r1) (ascending) in Ctx::pk with one warp; every thread gets
 // the count (-1: more than kBatch) and the largest end.  Ends with a barrier.
-__device__ __forceinline__ void list_long_gaps(const Ctx& c, int32_t r0, int32_t r1, Longs& lg, Shared& sh) {
+__device__ __forceinline__ void list_long_gaps(const Ctx<false>& c, int32_t r0, int32_t r1, Longs& lg, Shared& sh) {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     if (threadIdx.x == 0) sh.best32 = 0xffffffffu;
@@ -916,7 +985,7 @@ __device__ __forceinline__ void list_long_gaps(const Ctx& c, int32_t r0, int32_t
 // each tensor taking the bottom of its gap.  (40 tensors that span a trace of
 // 2,000, in 4 groups: 280 K cycles one by one, 120 K in groups.)  Returns false, with nothing placed, if there are more
 // than kBatch such gaps; ends with a barrier.
-__device__ __forceinline__ bool place_group(const Ctx& c, int32_t r, int32_t g, int32_t len, int32_t nlp, Shared& sh,
+__device__ __forceinline__ bool place_group(const Ctx<false>& c, int32_t r, int32_t g, int32_t len, int32_t nlp, Shared& sh,
                                             uint32_t* end) {
     const int32_t t = (int32_t)threadIdx.x, nt = (int32_t)blockDim.x;
     const unsigned full = 0xffffffffu;
@@ -1037,7 +1106,7 @@ __device__ __forceinline__ bool place_group(const Ctx& c, int32_t r, int32_t g, 
 // Places every tensor of ranks [0, n): runs of short tensors between the long
 // ones, whose ranks are lr[0, nl), ascending.  Returns the largest end this
 // thread knows of.
-__device__ __forceinline__ uint32_t place_all(const Ctx& c, int32_t n, const uint16_t* lr, int32_t nl, Shared& sh) {
+__device__ __forceinline__ uint32_t place_all(const Ctx<false>& c, int32_t n, const uint16_t* lr, int32_t nl, Shared& sh) {
     uint32_t mx = 0;
     int32_t r0 = 0, len = 0, pending = 0;  // ranks [pending, r0) are placed but not in the sorted list
     Longs lg = {0, -1, 0, 0xffffffffu, 0};
@@ -1299,7 +1368,7 @@ __device__ __forceinline__ bool plan(const mp_batch& bt, const TraceView& tv, in
         x.pos = (uint16_t)p;
         x.next = kNone;
         x.prev = (int32_t)x.f - (int32_t)x.a > kLong ? kIsLong : kNone;
-        x.pad = 0;
+        x.many = 0;
         REC[r] = x;
         TMP[p] = (uint16_t)r;
     }
@@ -1401,11 +1470,11 @@ __device__ __forceinline__ bool plan(const mp_batch& bt, const TraceView& tv, in
         if (flag && at < (uint32_t)kMaxLong) LR[at] = (uint16_t)r;
         nl += (int32_t)tot;
     }
-    if (nl > kMaxLong) return false;
+    if (nl > kMaxLong || (nl > 0 && sh.far > kLongestChain)) return false;
     for (int32_t p = t; p < n; p += nt) OE[p] = make_uint2(0, 0);
     __syncthreads();
 
-    Ctx c;
+    Ctx<false> c = {};
     c.oe = OE;
     c.af = AF;
     c.sl = SL;

@@ -88,3 +88,62 @@ def test_phases_limits(cuda_lib, case):
         else:  # every short-lived tensor in one chain, windows past 64 positions
             traces.append(_trace(rng, 1500, 300, 0.02, 64, 1 << 12, life=30, full_span=full))
     _check(tg.from_arrays(traces))
+
+
+def _far_trace(rng, n, T, kind):
+    a = rng.integers(0, T, n)
+    f = a + rng.integers(1, 6, n)
+    s = rng.integers(1, 1 << 16, n) * 64
+    far = rng.random(n) < 0.05
+    if kind == "long-tail":
+        f = np.where(far, a + rng.integers(100, T // 2 + 1, n), f)
+    elif kind == "full-span":  # groups of one lifetime, few sizes
+        a, f = np.where(far, 0, a), np.where(far, T, f)
+        s = rng.choice([64, 4096, 1 << 20], n)
+    elif kind == "crowded-steps":  # over kEdges tensors just before a long one's start, chains past kNear neighbours
+        a[: 1500] = rng.integers(10, 14, 1500)
+        f = a + rng.integers(1, 6, n)
+        f[:4] = a[:4] + 60
+        a[4:8], f[4:8] = 16, T
+    elif kind == "wide-sums":  # past 2^32 units: the dataflow
+        s[0], s[1] = (1 << 35) + 1, 1
+    elif kind == "short-only":
+        pass
+    elif kind == "all-long":
+        f = a + 33 + rng.integers(0, 40, n)
+        far[:] = True
+    return T, a, np.minimum(f, T), s
+
+
+@pytest.mark.parametrize("kind,n", (("long-tail", 5000), ("long-tail", 20000), ("full-span", 6001), ("crowded-steps", 7000),
+                                    ("wide-sums", 4500), ("short-only", 23000), ("short-only", 24000),
+                                    ("all-long", 4200), ("mixed", 9000), ("phased", 9000)))
+def test_large_traces_in_phases(cuda_lib, kind, n):
+    """One large trace per SM (batches of a few, past what one CTA prepares in
+    its shared memory), and those left to the grid-wide dataflow."""
+    import paper_2203_00448_gb300 as mp
+
+    rng = np.random.default_rng(n + len(kind))
+    kinds = {"mixed": ("long-tail", "full-span", "wide-sums", "short-only"),
+             "phased": ("long-tail", "full-span", "long-tail")}.get(kind, (kind,))
+    traces = [_far_trace(rng, n, n // 2 + 100, k) for k in kinds]
+    if kind in ("mixed", "phased"):
+        traces += [(10, np.zeros(0, np.int64), np.zeros(0, np.int64), np.zeros(0, np.int64)),
+                   (9, np.array([0, 3]), np.array([4, 2]), np.array([8, 8])),  # free <= alloc
+                   _far_trace(rng, 300, 200, "short-only")]
+    ts = tg.from_arrays(traces)
+    db = mp.DeviceBatch.from_host(ts, "cuda")
+    o_prof, o_lb, _ = oracle.live_profile(ts)
+    for policy, pol in (("first", oracle.FIT_FIRST), ("best", oracle.FIT_BEST)):
+        o_off, o_pk, o_st = oracle.plan_greedy_by_size(ts, pol)
+        r = mp.plan_and_validate(db, policy)
+        off, pk, st = mp.plan_greedy_by_size(db, policy)
+        st, rst = st.cpu().numpy(), r.status.cpu().numpy()
+        assert st.tolist() == o_st.tolist() == rst.tolist()
+        for b in np.flatnonzero(o_st == 0):
+            lo, hi = ts.trace_ptr[b], ts.trace_ptr[b + 1]
+            assert np.array_equal(off[lo:hi].cpu().numpy(), o_off[lo:hi]), (policy, b)
+            assert np.array_equal(r.offsets[lo:hi].cpu().numpy(), o_off[lo:hi]), (policy, b)
+            assert int(pk[b]) == o_pk[b] == int(r.plan_peak[b]) and int(r.verdict[b]) == 1
+            plo, phi = ts.profile_ptr[b], ts.profile_ptr[b + 1]
+            assert np.array_equal(r.profile[plo:phi].cpu().numpy(), o_prof[plo:phi]) and int(r.peak_lb[b]) == o_lb[b]
