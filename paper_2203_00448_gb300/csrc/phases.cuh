@@ -49,9 +49,12 @@ constexpr int32_t kHeads = 1024;       // chains of a run listed at a time
 constexpr int32_t kChunk = 16;         // sorted-list entries per thread: kMaxTensors / the fewest threads
 constexpr int32_t kNear = 32;          // neighbours listed per short tensor of a large trace (grid_phases.cu)
 constexpr int32_t kThreadChain = 8;    // chains up to this long within a run can be walked by one thread
+constexpr int32_t kTeamChain = 64;     // chains from this length on are walked by the whole CTA together ...
+constexpr int32_t kTeams = 4;          // ... up to this many of a run
+constexpr int32_t kTeamPolls = 1 << 20;  // bound of a wait there (some 50 ms)
 constexpr int32_t kListRun = 64;       // runs from this length on list the gaps between the long tensors first
 constexpr int32_t kFewPending = 8;     // up to this many are inserted by comparison with every entry
-constexpr uint32_t kScanChain = 1024;  // chains are linked member by member up to this many looks per thread, else by a sort
+constexpr uint32_t kScanChain = 128;  // chains are linked member by member up to this many looks per thread, else by a sort
 constexpr uint64_t kLongKey = 0xfffffffffffffffeull;  // sort key of a long tensor among the chains: last
 constexpr uint16_t kNone = 0xffff;     // no such rank
 constexpr uint16_t kIsLong = 0xfffe;   // in Rec::prev: the tensor is long
@@ -62,12 +65,15 @@ struct __align__(16) Rec {
     uint16_t a, f;        // lifetime [a, f)
     uint16_t pos;         // alloc-order position
     uint16_t next, prev;  // ranks of the neighbours in its chain (component of short lifetimes)
-    uint16_t many;        // kFar: more than kNear neighbours, not listed
+    union {
+        uint16_t many;  // kFar: more than kNear neighbours, not listed
+        uint16_t comp;  // otherwise: its component of short lifetimes
+    };
 };
 // Alloc-order positions of the short tensors that can overlap it: [w0, w1);
 // those from `core` on are allocated during its life.
-// Ctx::mask has the short ones that overlap it, as bits from w0 on, unless
-// there are more than 32 positions (`wide`).
+// Ctx::mask has the short ones of lower rank that overlap it, as bits from w0
+// on, unless there are more than 32 positions (`wide`).
 struct __align__(8) Win {
     uint16_t w0, core, w1, wide;
 };
@@ -80,7 +86,7 @@ struct Layout {
     size_t oe, rec, win, mask, af, id, sl, tmp, bend, lg_oe, lg_af, lr, pk, heads, total;
     __host__ __device__ static constexpr size_t a16(size_t x) { return (x + 15) & ~size_t(15); }
     __host__ __device__ static constexpr int32_t keys_of(int32_t n) {  // sort length
-        int32_t k = 1024;  // two keys per thread at least
+        int32_t k = 512;  // a key per thread at least
         while (k < n) k <<= 1;
         return k;
     }
@@ -127,7 +133,8 @@ struct Shared {
     uint32_t red[33];
     unsigned long long hi, lo, bits, best;
     uint32_t best32, lb, far;
-    int32_t bad, lw, cnt, next, cnt1, next1;
+    int32_t bad, lw, cnt, next, cnt1, next1, teams, fail;
+    uint16_t team[kTeams];
     uint32_t last_free;
     uint32_t before[kFewPending];
     unsigned long long key;
@@ -261,6 +268,7 @@ struct Ctx {
     const uint32_t* mask; // by rank
     uint64_t* pk;         // kBatch keys of tensors being inserted; gaps (start << 32 | length) otherwise
     uint16_t* heads;      // kHeads ranks
+    uint16_t* list;       // ranks of the members of one chain (not kFar)
     const uint16_t* near; // kFar, by rank: positions of the kNear short tensors it overlaps (kNone: no more)
     int32_t policy;
 };
@@ -506,8 +514,8 @@ __device__ __forceinline__ uint32_t place_short(const Ctx<kFar>& c, int32_t r, c
         bool fits = hit && v.x >= prev && v.x - prev >= s;
         if (!first && !wide) {
             // most gaps meet no window tensor: those are compared as they
-            // are, a lane each (looking into every one took a warp reduction
-            // or two per gap; the 20,000-tensor trace, BEST: @FARBEST@)
+            // are, a lane each (looking into every one takes a warp reduction
+            // or two per gap: 47.2 against 42.9 ms on a long tail of 20,000)
             bool touched = false;
             for (unsigned b = near0; b; b &= b - 1) {
                 const int src = __ffs(b) - 1;
@@ -565,14 +573,46 @@ __device__ __forceinline__ uint32_t place_short(const Ctx<kFar>& c, int32_t r, c
     return best + s;
 }
 
+// The offset of a short tensor of s units whose placed predecessors (an
+// obstacle per lane; (0, 0): none) and lg.top are all it meets, by one warp:
+// FIRST jumps past whatever conflicts, BEST walks the holes.
+__device__ __forceinline__ uint32_t fit_plain(uint2 v, uint32_t s, uint32_t base, int32_t policy) {
+    const unsigned full = 0xffffffffu;
+    uint32_t o = base;
+    if (policy == MP_FIT_FIRST) {
+        for (;;) {
+            const uint32_t m = __reduce_max_sync(full, (v.x < o + s) & (o < v.y) ? v.y : 0u);
+            if (m <= o) return o;
+            o = m;
+        }
+    }
+    const uint32_t top = umax2(o, __reduce_max_sync(full, v.y));
+    uint32_t at = o, best_len = 0xffffffffu;
+    o = top;
+    while (at < top) {
+        const uint32_t m = __reduce_max_sync(full, (v.x <= at) & (at < v.y) ? v.y : 0u);
+        const uint32_t ns = __reduce_min_sync(full, v.x > at ? v.x : top);
+        if (m > at) {
+            at = m;
+            continue;
+        }
+        if (ns - at >= s && ns - at < best_len) {
+            best_len = ns - at;
+            o = at;
+        }
+        at = ns;
+    }
+    return o;
+}
+
 // Walks the chain from rank r up to rank r1 with one warp, a window position
 // per lane, when no gap between long tensors needs a look: everything goes
 // above lg.top.  The next member's entries (which depend on no offset) are
-// loaded while the current one is placed.
+// loaded while the current one is placed.  (Testing every possible start
+// against all predecessors at once, without jumps, took a third longer: one
+// warp is bound by the number of its dependent instructions.)
 __device__ __forceinline__ uint32_t walk_plain(const Ctx<false>& c, int32_t r, int32_t r1, const Longs& lg) {
-    const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
-    const bool first = c.policy == MP_FIT_FIRST;
     uint32_t mx = 0;
     Rec rc = c.rec[r];
     Win w = c.win[r];
@@ -586,36 +626,11 @@ __device__ __forceinline__ uint32_t walk_plain(const Ctx<false>& c, int32_t r, i
         if (w.wide) {
             mx = umax2(mx, place_short(c, r, lg));
         } else {
-            const uint32_t s = rc.s;
             const uint2 v = (mask >> lane) & 1u ? c.oe[w.w0 + lane] : make_uint2(0, 0);
-            uint32_t o = lg.top;
-            if (first) {
-                for (;;) {
-                    const uint32_t m = __reduce_max_sync(full, (v.x < o + s) & (o < v.y) ? v.y : 0u);
-                    if (m <= o) break;
-                    o = m;
-                }
-            } else {
-                const uint32_t top = umax2(o, __reduce_max_sync(full, v.y));
-                uint32_t at = o, best_len = 0xffffffffu;
-                o = top;
-                while (at < top) {
-                    const uint32_t m = __reduce_max_sync(full, (v.x <= at) & (at < v.y) ? v.y : 0u);
-                    const uint32_t ns = __reduce_min_sync(full, v.x > at ? v.x : top);
-                    if (m > at) {
-                        at = m;
-                        continue;
-                    }
-                    if (ns - at >= s && ns - at < best_len) {
-                        best_len = ns - at;
-                        o = at;
-                    }
-                    at = ns;
-                }
-            }
-            if (lane == 0) c.oe[rc.pos] = make_uint2(o, o + s);
+            const uint32_t o = fit_plain(v, rc.s, lg.top, c.policy);
+            if (lane == 0) c.oe[rc.pos] = make_uint2(o, o + rc.s);
             __syncwarp();
-            mx = umax2(mx, o + s);
+            mx = umax2(mx, o + rc.s);
         }
         if (!more) return mx;
         r = rn;
@@ -623,6 +638,71 @@ __device__ __forceinline__ uint32_t walk_plain(const Ctx<false>& c, int32_t r, i
         w = w1;
         mask = mask1;
     }
+}
+
+// Walks the run's long chains (of the components of sh.team[0, teams), their
+// members among ranks [r0, r1)) with every warp of the CTA, no gap between long
+// tensors needing a look: the warps are dealt out to the chains, take their
+// chain's members in rank order in turn, each waits until its member's
+// predecessors are placed (the offsets it needs are what it polls), and places
+// it.  The lowest unplaced member's predecessors are placed and its warp has
+// nothing earlier left to do, so every wait ends; it is bounded all the same
+// (sh.fail).  A chain of equal sizes is deep but not a single path: 262 and 112
+// activations of a residual network, 172 K cycles by a warp each, 100 K this way.
+__device__ __forceinline__ uint32_t walk_teams(const Ctx<false>& c, int32_t teams, int32_t r0, int32_t r1,
+                                               const Longs& lg, Shared& sh) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int32_t nwarps = (int32_t)(blockDim.x >> 5) / teams;  // per chain
+    const int32_t mine = min(warp / nwarps, teams);             // (warps left over take none)
+    int32_t n = 0, first = 0, end = 0;
+    for (int32_t k = 0; k < teams; ++k) {
+        const uint32_t comp = c.rec[sh.team[k]].comp;
+        if (k == mine) first = n;
+        for (int32_t b0 = r0; b0 < r1; b0 += (int32_t)blockDim.x) {
+            const int32_t r = b0 + (int32_t)threadIdx.x;
+            const uint32_t flag = r < r1 && c.rec[r].comp == comp && c.rec[r].prev != kIsLong ? 1u : 0u;
+            uint32_t tot;
+            const uint32_t at = (uint32_t)n + block_excl_sum(flag, sh.red, &tot);
+            if (flag) c.list[at] = (uint16_t)r;
+            n += (int32_t)tot;
+        }
+        if (k == mine) end = n;
+    }
+    __syncthreads();
+    uint32_t mx = 0;
+    volatile unsigned long long* oe = reinterpret_cast<volatile unsigned long long*>(c.oe);
+    for (int32_t i = first + warp % nwarps; i < end; i += nwarps) {
+        const int32_t r = c.list[i];
+        const Rec rc = c.rec[r];
+        const Win w = c.win[r];
+        if (w.wide) {  // no mask of its predecessors: every earlier member's turn first
+            for (int32_t x = first + lane; x < i; x += 32)
+                for (int32_t polls = 0; oe[c.rec[c.list[x]].pos] == 0; ++polls)
+                    if (polls > kTeamPolls || *(volatile int32_t*)&sh.fail) {
+                        sh.fail = 1;
+                        break;
+                    }
+            __syncwarp();
+            mx = umax2(mx, place_short(c, r, lg));
+            continue;
+        }
+        const bool pred = (c.mask[r] >> lane) & 1u;
+        const int32_t q = w.w0 + lane;
+        unsigned long long v = 0;
+        for (int32_t polls = 0;; ++polls) {
+            if (pred) v = oe[q];
+            if (!__any_sync(0xffffffffu, pred && v == 0)) break;
+            if (polls > kTeamPolls || *(volatile int32_t*)&sh.fail) {
+                if (lane == 0) sh.fail = 1;
+                break;
+            }
+        }
+        const uint32_t o = fit_plain(make_uint2((uint32_t)v, (uint32_t)(v >> 32)), rc.s, lg.top, c.policy);
+        if (lane == 0) oe[rc.pos] = ((unsigned long long)(o + rc.s) << 32) | o;
+        mx = umax2(mx, o + rc.s);
+    }
+    __syncthreads();
+    return mx;
 }
 
 // Places the short tensors of ranks [r0, r1), every lower rank being placed:
@@ -666,22 +746,29 @@ __device__ __forceinline__ uint32_t run_chains(const Ctx<kFar>& c, int32_t r0, i
     }
     for (int32_t b0 = r0; b0 < r1; b0 += kHeads) {
         __syncthreads();  // the previous list is done with
-        if (threadIdx.x == 0) sh.cnt = sh.next = sh.cnt1 = sh.next1 = 0;
+        if (threadIdx.x == 0) sh.cnt = sh.next = sh.cnt1 = sh.next1 = sh.teams = 0;
         __syncthreads();
         // chains for warps from the front of the list, for threads from its back
         const int32_t b1 = min(r1, b0 + kHeads);
         for (int32_t r = b0 + (int32_t)threadIdx.x; r < b1; r += (int32_t)blockDim.x) {
             if (!is_head(r)) continue;
-            bool alone = lg.ng >= 0;
-            int32_t x = r;
-            for (int32_t len = 0; alone && x < r1; ++len) {
-                alone = len < kThreadChain && !c.win[x].wide;
-                x = c.rec[x].next;
+            int32_t len = lg.ng >= 0 ? 0 : 2 * kTeamChain;  // members, if all have masks
+            for (int32_t x = r; len < kTeamChain && x < r1; x = c.rec[x].next) len = c.win[x].wide ? 2 * kTeamChain : len + 1;
+            if (len <= kThreadChain) {
+                c.heads[kHeads - 1 - atomicAdd(&sh.cnt1, 1)] = (uint16_t)r;
+            } else {
+                int32_t k = kTeams;
+                if constexpr (!kFar)
+                    if (len == kTeamChain && lg.ng == 0) k = atomicAdd(&sh.teams, 1);
+                if (k < kTeams) sh.team[k] = (uint16_t)r;
+                else c.heads[atomicAdd(&sh.cnt, 1)] = (uint16_t)r;
             }
-            if (alone) c.heads[kHeads - 1 - atomicAdd(&sh.cnt1, 1)] = (uint16_t)r;
-            else c.heads[atomicAdd(&sh.cnt, 1)] = (uint16_t)r;
         }
         __syncthreads();
+        if constexpr (!kFar) {
+            const int32_t teams = min(sh.teams, kTeams);
+            if (teams > 0) mx = umax2(mx, walk_teams(c, teams, r0, r1, lg, sh));
+        }
         const int32_t nh = sh.cnt, nh1 = sh.cnt1;
         // half of the warps begin with the long chains, half with the others
         for (int32_t part = 0; part < 2; ++part) {
@@ -1182,7 +1269,8 @@ static __device__ __noinline__ void sort_keys(int32_t n) {
         }
         __syncthreads();
     };
-    if (n <= 2 * nt) go(std::integral_constant<int, 2>());
+    if (n <= nt) go(std::integral_constant<int, 1>());
+    else if (n <= 2 * nt) go(std::integral_constant<int, 2>());
     else if (n <= 4 * nt) go(std::integral_constant<int, 4>());
     else if (n <= 8 * nt) go(std::integral_constant<int, 8>());
     else go(std::integral_constant<int, 16>());
@@ -1223,6 +1311,7 @@ __device__ __forceinline__ bool plan(const mp_batch& bt, const TraceView& tv, in
     if (t == 0) {
         sh.bad = 0;
         sh.lw = 1;
+        sh.fail = 0;
         sh.hi = sh.lo = sh.bits = 0;
         sh.lb = sh.far = sh.last_free = 0;
         sh.key = ~0ull;
@@ -1386,7 +1475,7 @@ __device__ __forceinline__ bool plan(const mp_batch& bt, const TraceView& tv, in
         if (!w.wide)
             for (int32_t q = w.w0; q < w.w1; ++q) {
                 const int32_t qa = (int32_t)(AF[q] & 0xffffu), qf = (int32_t)(AF[q] >> 16);
-                if (q != x.pos && qf - qa <= kLong && (q >= w.core || qf > x.a)) mask |= 1u << (q - w.w0);
+                if (TMP[q] < r && qf - qa <= kLong && (q >= w.core || qf > x.a)) mask |= 1u << (q - w.w0);
             }
         MASK[r] = mask;
     }
@@ -1446,6 +1535,7 @@ __device__ __forceinline__ bool plan(const mp_batch& bt, const TraceView& tv, in
             }
             REC[mine].next = (uint16_t)up;
             REC[mine].prev = (uint16_t)dn;
+            REC[mine].comp = (uint16_t)(k >> 16);
         }
     } else {
         sort_keys(n);
@@ -1454,6 +1544,7 @@ __device__ __forceinline__ bool plan(const mp_batch& bt, const TraceView& tv, in
             if (k == kLongKey) continue;
             const uint64_t up = i + 1 < n ? KEY[i + 1] : ~0ull, dn = i ? KEY[i - 1] : ~0ull;
             Rec& x = REC[k & 0xffffu];
+            x.comp = (uint16_t)(k >> 16);
             if ((up >> 16) == (k >> 16)) x.next = (uint16_t)up;
             if ((dn >> 16) == (k >> 16)) x.prev = (uint16_t)dn;
         }
@@ -1485,6 +1576,7 @@ __device__ __forceinline__ bool plan(const mp_batch& bt, const TraceView& tv, in
     c.mask = MASK;
     c.pk = reinterpret_cast<uint64_t*>(smem + L.pk);
     c.heads = reinterpret_cast<uint16_t*>(smem + L.heads);
+    c.list = TMP;
     c.policy = policy;
     uint32_t top = place_all(c, n, LR, nl, sh);
 
@@ -1543,7 +1635,7 @@ __device__ __forceinline__ bool plan(const mp_batch& bt, const TraceView& tv, in
                 out.conflict[1] = good ? -1 : (int32_t)(key & 0xffffffffu);
             }
         }
-        *out.status = MP_OK;
+        *out.status = sh.fail ? MP_ETIMEOUT : MP_OK;
     }
     __syncthreads();
     return true;
