@@ -12,13 +12,14 @@ namespace mp {
 
 constexpr int kProfileThreads = 128;  // one CTA per trace
 constexpr int kValidateThreads = 128;
-constexpr int kPeakThreads = 256;
+constexpr int kPeakThreads = 128;
 constexpr int kBumpThreads = 128;
 constexpr int kOptThreads = 128;
 constexpr int kReplayThreads = 256;
 constexpr int kBreadthThreads = 128;
 constexpr int kBreadthPhaseThreads = 512;  // half of it when the batch has more traces than the GPU SMs
 constexpr int kPlanThreadsSmem = 128;    // one CTA per trace, data in shared memory
+constexpr int kPlanThreadsFew = 512;     // ... in a batch of few traces
 constexpr int kPlanThreadsGlobal = 1024; // one CTA per trace, data in the workspace
 constexpr int kPlanThreadsWide = 512;    // the 64-bit launch: deferred traces, CTA tier included
 

@@ -31,8 +31,8 @@
 //     the component into priority order and place it by a ready queue (runs of
 //     short-lived tensors) and CTA-wide gap searches (long-lived ones).  256
 //     traces of 2,000 tensors with 40 that span the trace, fused, best fit: 7.9
-//     ms by queue, 0.37 ms in phases; a chain of 374 activations: 133 us walked
-//     by the first launch's 128 threads, 120 us in phases.
+//     ms by queue, 0.37 ms in phases; a chain of 374 activations: 136 us walked
+//     by the first launch's 128 threads, 85 us in phases.
 // Thread-tier components are handed out largest size class first, so the
 // lanes of a warp carry similar work.
 //
@@ -78,6 +78,8 @@ namespace {
 // tensors: 110.8 us with 9 (52 registers), 110.7 with 10 (48), 113.7 with 12
 // (40, spills); 301 ragged ones, best fit: 39.7, 40.2 and 41.7 us.
 constexpr int kPlanCtasSmem = 9;
+constexpr int32_t kFewTensors = 256;   // batches of few traces: longer ones than this get kPlanThreadsFew threads
+constexpr int32_t kSmallSteps = 2048;  // steps of a small trace (k_plan_small): four CTAs' working sets fit an SM
 constexpr int32_t kThreadComp = 8;   // components up to this size: one thread
 constexpr int32_t kWarpComp = 64;    // ... up to this size: one warp (a tensor or two per lane); else the CTA
 constexpr int kCached = 4;           // tensors per thread kept in registers between the two input passes
@@ -1436,7 +1438,7 @@ __device__ __forceinline__ int32_t test_hold_position(int) { return -1; }
 // ------------------------------------------------------------- the kernel
 
 // The whole path for trace b, by the whole CTA.
-template <typename I, typename W, bool kSmem, bool kFused>
+template <typename I, typename W, bool kSmem, bool kFused, bool kCtaTier>
 __device__ __forceinline__ void plan_trace(const int b, const mp_batch& bt, const PlanOut& out,
                                            unsigned char* __restrict__ ws, size_t data_stride, size_t buf_offset,
                                            size_t buf_stride) {
@@ -1797,7 +1799,7 @@ __device__ __forceinline__ void plan_trace(const int b, const mp_batch& bt, cons
     }
 
     // ---- large components, the whole CTA each
-    if constexpr (kWide) if (s_base[kBins] > s_base[kBinCta]) {
+    if constexpr (kCtaTier) if (s_base[kBins] > s_base[kBinCta]) {
         const W e = large_tier<I, W, kSmem>(AR, OFFP, BEND, SB, NW, LST + s_base[kBinCta], s_base[kBins] - s_base[kBinCta],
                                             n, ORD, HR, CNT,
                                             QUE, bo, be, smem_raw, policy, red, &s_cnt, &s_tail, &s_fail,
@@ -1896,9 +1898,8 @@ __device__ __forceinline__ bool plan_in_phases(const int b, const mp_batch& bt, 
 // what the GPU holds at once walks every trace and takes the ones the 32-bit
 // launch deferred (sizes summing to 2^32 or more, or a component the 32-bit
 // launch does not place), with larger CTAs for the CTA tier.
-template <typename I, typename W, bool kSmem, bool kFused>
-__global__ void __launch_bounds__(sizeof(W) == 8 ? kPlanThreadsWide : (kSmem ? kPlanThreadsSmem : kPlanThreadsGlobal),
-                                  sizeof(W) == 8 ? 1 : (kSmem ? kPlanCtasSmem : 1))
+template <typename I, typename W, bool kSmem, bool kFused, int kThreads>
+__global__ void __launch_bounds__(kThreads, sizeof(W) == 8 || !kSmem ? 1 : kThreads == kPlanThreadsFew ? 2 : kPlanCtasSmem)
 k_plan(mp_batch bt, PlanOut out, unsigned char* __restrict__ ws, size_t data_stride, size_t buf_offset,
        size_t buf_stride, bool in_phases) {
     if constexpr (sizeof(W) == 4) {
@@ -1906,7 +1907,7 @@ k_plan(mp_batch bt, PlanOut out, unsigned char* __restrict__ ws, size_t data_str
         // what room is left; they wait for this grid to finish (and its writes
         // to land) before they read anything it wrote
         asm volatile("griddepcontrol.launch_dependents;");
-        plan_trace<I, W, kSmem, kFused>(blockIdx.x, bt, out, ws, data_stride, buf_offset, buf_stride);
+        plan_trace<I, W, kSmem, kFused, false>(blockIdx.x, bt, out, ws, data_stride, buf_offset, buf_stride);
     } else {
         asm volatile("griddepcontrol.wait;" ::: "memory");
         // this CTA's traces are blockIdx.x + k * gridDim.x; their statuses are
@@ -1924,12 +1925,26 @@ k_plan(mp_batch bt, PlanOut out, unsigned char* __restrict__ ws, size_t data_str
             while (m) {
                 const int b = (int)(blockIdx.x + (k0 + __ffs(m) - 1) * gridDim.x);
                 m &= m - 1;
-                if (!in_phases || !plan_in_phases<kFused>(b, bt, out))
-                    plan_trace<I, W, kSmem, kFused>(b, bt, out, ws, data_stride, buf_offset, buf_stride);
+                bool done = false;
+                if constexpr (sizeof(I) == 2) done = in_phases && plan_in_phases<kFused>(b, bt, out);
+                if (!done)
+                    plan_trace<I, W, kSmem, kFused, true>(b, bt, out, ws, data_stride, buf_offset, buf_stride);
                 __syncthreads();
             }
         }
     }
+}
+
+// Small traces (at most kWarpComp tensors, so no large component) in a batch of
+// few: the 32-bit pass, and the 64-bit one for a trace whose sizes need it, in
+// one launch.
+template <bool kFused>
+__global__ void __launch_bounds__(kPlanThreadsSmem, 4) k_plan_small(mp_batch bt, PlanOut out) {
+    const int b = blockIdx.x;
+    plan_trace<int16_t, uint32_t, true, kFused, false>(b, bt, out, nullptr, 0, 0, 0);
+    __syncthreads();
+    if (*(volatile int32_t*)(out.status + b) != kDeferred) return;
+    plan_trace<int16_t, int64_t, true, kFused, false>(b, bt, out, nullptr, 0, 0, 0);
 }
 
 struct PlanGeometry {
@@ -1972,12 +1987,12 @@ PlanWorkspace plan_workspace(const mp_batch& bt) {
     return w;
 }
 
-template <typename I, typename W, bool kSmem, bool kFused>
+template <typename I, typename W, bool kSmem, bool kFused, int kThreads>
 cudaError_t launch_variant(const mp_batch& bt, const PlanGeometry& g, const PlanWorkspace& pw, const PlanOut& out,
                            unsigned char* ws, cudaStream_t stream) {
-    int threads = sizeof(W) == 8 ? kPlanThreadsWide : (kSmem ? kPlanThreadsSmem : kPlanThreadsGlobal);
+    int threads = kThreads;
     size_t smem = kSmem ? g.data : (sizeof(W) == 8 ? flow_smem_bytes<W>() : 0);
-    const bool in_phases = sizeof(W) == 8 && phases::batch_fits<false>(bt);
+    const bool in_phases = sizeof(W) == 8 && sizeof(I) == 2 && phases::batch_fits<false>(bt);
     if (in_phases) {
         smem = std::max(smem, phases::smem_bytes<false>(bt));
         // more traces than SMs: half the threads, so that an SM holds two
@@ -1986,7 +2001,7 @@ cudaError_t launch_variant(const mp_batch& bt, const PlanGeometry& g, const Plan
         if (e != cudaSuccess) return e;
         if (bt.n_traces > sms) threads /= 2;
     }
-    const void* fn = (const void*)k_plan<I, W, kSmem, kFused>;
+    const void* fn = (const void*)k_plan<I, W, kSmem, kFused, kThreads>;
     {
         cudaError_t e = set_smem_limit(fn, smem);
         if (e != cudaSuccess) return e;
@@ -1999,7 +2014,7 @@ cudaError_t launch_variant(const mp_batch& bt, const PlanGeometry& g, const Plan
         grid = std::max(1, std::min(grid, resident));
     }
     if (sizeof(W) == 4) {
-        k_plan<I, W, kSmem, kFused><<<(unsigned)grid, threads, smem, stream>>>(
+        k_plan<I, W, kSmem, kFused, kThreads><<<(unsigned)grid, threads, smem, stream>>>(
             bt, out, ws, g.data_stride, pw.buf_offset, pw.buf_stride, false);
         return cudaGetLastError();
     }
@@ -2015,7 +2030,7 @@ cudaError_t launch_variant(const mp_batch& bt, const PlanGeometry& g, const Plan
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_plan<I, W, kSmem, kFused>, bt, out, ws, g.data_stride, pw.buf_offset,
+    return cudaLaunchKernelEx(&cfg, k_plan<I, W, kSmem, kFused, kThreads>, bt, out, ws, g.data_stride, pw.buf_offset,
                               pw.buf_stride, in_phases);
 }
 
@@ -2023,16 +2038,44 @@ template <typename W, bool kFused>
 cudaError_t launch_width(const mp_batch& bt, const PlanOut& out, unsigned char* ws, cudaStream_t stream) {
     const PlanGeometry g = plan_geometry<W>(bt, kFused);
     const PlanWorkspace pw = plan_workspace(bt);
+    constexpr int kSmemThreads = sizeof(W) == 8 ? kPlanThreadsWide : kPlanThreadsSmem;
+    constexpr int kGlobalThreads = sizeof(W) == 8 ? kPlanThreadsWide : kPlanThreadsGlobal;
+    if constexpr (sizeof(W) == 4) {
+        // traces of some length, too few to fill the GPU with 128 threads each:
+        // the latency of one CTA is what counts, and more threads shorten all
+        // but the placement of its longest component (301 ragged traces of up
+        // to 701 tensors, best fit: 39.7 us with 128 threads, 31.1 with 512)
+        int sms = 0;
+        const cudaError_t e = sm_count(&sms);
+        if (e != cudaSuccess) return e;
+        if (g.narrow && g.smem && bt.max_tensors > kFewTensors && bt.n_traces <= 2 * sms)
+            return launch_variant<int16_t, W, true, kFused, kPlanThreadsFew>(bt, g, pw, out, ws, stream);
+    }
     if (g.narrow)
-        return g.smem ? launch_variant<int16_t, W, true, kFused>(bt, g, pw, out, ws, stream)
-                      : launch_variant<int16_t, W, false, kFused>(bt, g, pw, out, ws, stream);
-    return g.smem ? launch_variant<int32_t, W, true, kFused>(bt, g, pw, out, ws, stream)
-                  : launch_variant<int32_t, W, false, kFused>(bt, g, pw, out, ws, stream);
+        return g.smem ? launch_variant<int16_t, W, true, kFused, kSmemThreads>(bt, g, pw, out, ws, stream)
+                      : launch_variant<int16_t, W, false, kFused, kGlobalThreads>(bt, g, pw, out, ws, stream);
+    return g.smem ? launch_variant<int32_t, W, true, kFused, kSmemThreads>(bt, g, pw, out, ws, stream)
+                  : launch_variant<int32_t, W, false, kFused, kGlobalThreads>(bt, g, pw, out, ws, stream);
 }
 
 template <bool kFused>
 cudaError_t launch_any(const mp_batch& bt, const PlanOut& out, void* workspace, cudaStream_t stream) {
     if (bt.n_traces == 0) return cudaSuccess;
+    if (bt.max_tensors <= kWarpComp) {
+        // one launch instead of two (one trace of 64 tensors: 26 us a call,
+        // 22 so, the host's part being most of it); with more traces than the GPU
+        // holds at once, the leaner kernel of the first launch is the faster one
+        const size_t smem = PlanLayout<int16_t, int64_t>(bt.max_tensors, bt.max_steps, kFused).total;
+        int sms = 0;
+        cudaError_t e = sm_count(&sms);
+        if (e != cudaSuccess) return e;
+        if (bt.max_steps <= kSmallSteps && bt.n_traces <= 4 * sms) {
+            e = set_smem_limit((const void*)k_plan_small<kFused>, smem);
+            if (e != cudaSuccess) return e;
+            k_plan_small<kFused><<<(unsigned)bt.n_traces, kPlanThreadsSmem, smem, stream>>>(bt, out);
+            return cudaGetLastError();
+        }
+    }
     unsigned char* ws = static_cast<unsigned char*>(workspace);
     cudaError_t e = launch_width<uint32_t, kFused>(bt, out, ws, stream);
     if (e != cudaSuccess) return e;
