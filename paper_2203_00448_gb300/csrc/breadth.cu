@@ -10,21 +10,20 @@
 // operator's step (the earlier on ties), then size descending, alloc step
 // ascending, id ascending.
 //
-// GPU form: one CTA per trace, in up to three kernels.  k_breadth_comp places
-// every trace whose working set fits in shared memory by lifetime components
-// (see its comment below): a thread, a warp or the whole CTA per component.
-// The traces it leaves (a component past kBBigComp tensors, or too many of its
-// large ones) go to k_breadth_phases, which places a trace's short-lived
-// tensors by chains and its long-lived ones by the whole CTA over a list
-// sorted by offset (phases.cuh): 256 traces of 2,000 tensors take
-// 0.31 ms instead of 38.5 ms.
-// What that path does not take (sizes past 2^32 units, too many
-// long-lived tensors, traces past its limits) goes to k_breadth: the breadths
-// (two integer atomics per tensor, order-independent), each tensor's wider
-// operator, an in-place odd-even merge sort of the ids by that order, then
-// placement tensor by tensor: all warps gather the placed tensors whose
-// lifetimes overlap the next one (one shared counter update per warp) and warp
-// 0 runs the gap search with warp reductions.
+// GPU form: one CTA per trace, in two kernels.  k_breadth_comp places every
+// trace whose working set fits in shared memory by lifetime components (see its
+// comment below): a thread, a warp or the whole CTA per component.  The traces
+// it leaves (a component past kBBigComp tensors, or too many of its large ones)
+// go to k_breadth_rest, which places a trace's short-lived tensors by chains and
+// its long-lived ones by the whole CTA over a list sorted by offset
+// (phases.cuh): 256 traces of 2,000 tensors take 0.32 ms instead of 38.5 ms.
+// What that path does not take (sizes past 2^32 units, too many long-lived
+// tensors, traces past its limits) is placed there tensor by tensor
+// (breadth_trace): the breadths (two integer atomics per tensor, order-
+// independent), each tensor's wider operator, an in-place odd-even merge sort of
+// the ids by that order, then for each tensor all warps gather the placed
+// tensors whose lifetimes overlap it (one shared counter update per warp) and
+// warp 0 runs the gap search with warp reductions.
 #include <algorithm>
 
 #include "common.cuh"
@@ -35,7 +34,8 @@ namespace mp {
 
 namespace {
 
-constexpr int32_t kBDeferred = -2;  // status of a trace left by k_breadth_comp to k_breadth
+constexpr size_t kTwoPerSm = 110 * 1024;  // shared memory of a CTA of which an SM holds two
+constexpr int32_t kBDeferred = -2;  // status of a trace left by k_breadth_comp to k_breadth_rest
 
 // Per-trace working set: the breadth of the operator at each step; per tensor
 // (by id) its operator's breadth and step, (alloc, free), size and offset; the priority order; the
@@ -138,18 +138,18 @@ __device__ void block_sort_ids(int32_t* keys, int32_t n, Before&& before) {
     }
 }
 
+// Places trace b tensor by tensor with the whole CTA.
 template <bool kSmem>
-__global__ void __launch_bounds__(kBreadthThreads)
-k_breadth(mp_batch bt, int32_t policy, int64_t* __restrict__ offsets, int64_t* __restrict__ plan_peak,
-          int32_t* __restrict__ status, unsigned char* __restrict__ ws, size_t ws_stride, bool deferred_only) {
+__device__ __forceinline__ void breadth_trace(const int b, const mp_batch& bt, int32_t policy,
+                                              int64_t* __restrict__ offsets, int64_t* __restrict__ plan_peak,
+                                              int32_t* __restrict__ status, unsigned char* __restrict__ ws,
+                                              size_t ws_stride) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int64_t red[72];
     __shared__ int32_t s_cnt, s_bad;
     __shared__ unsigned long long s_hi, s_lo;
-    const int b = blockIdx.x;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
-    if (deferred_only && status[b] != kBDeferred) return;  // placed by k_breadth_comp
     const TraceView tv = load_trace(bt, b, false);
     if (tv.st != MP_OK) {
         if (threadIdx.x == 0) {
@@ -490,6 +490,9 @@ __device__ void place_comp_warp(const BRec* __restrict__ R, int64_t* __restrict_
 __global__ void __launch_bounds__(kBreadthThreads)
 k_breadth_comp(mp_batch bt, int32_t policy, int64_t* __restrict__ offsets, int64_t* __restrict__ plan_peak,
                int32_t* __restrict__ status, bool in_phases) {
+    // once every CTA of this grid runs, those of k_breadth_rest may take what
+    // room is left; they wait for this grid to finish
+    asm volatile("griddepcontrol.launch_dependents;");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int64_t red[72];
     __shared__ int32_t s_bad, s_defer, s_nt, s_nw, s_nb, s_cnt, s_bin[kBThreadComp - 1], s_base[kBThreadComp];
@@ -532,7 +535,7 @@ k_breadth_comp(mp_batch bt, int32_t policy, int64_t* __restrict__ offsets, int64
     }
     if (tid < kBThreadComp - 1) s_bin[tid] = 0;
     __syncthreads();
-    // checks, operator breadths (as in k_breadth) and the alloc-step histogram
+    // checks, operator breadths (as in breadth_trace) and the alloc-step histogram
     bool bad = false;
     uint64_t sum = 0;
     for (int32_t k = tid; k < n; k += nthr) {
@@ -744,29 +747,99 @@ k_breadth_comp(mp_batch bt, int32_t policy, int64_t* __restrict__ offsets, int64
     }
 }
 
-// The deferred traces (or, with deferred_only false, all of them) in phases;
-// those it does not take are left deferred.
+// The traces k_breadth_comp deferred (or, with deferred_only false, all of
+// them), in phases where they fit that path (in_phases: the batch may), else
+// tensor by tensor (by_tensor; otherwise they are left deferred).  It waits for
+// the kernel before it in the kernel.
+template <bool kSmem>
 __global__ void __launch_bounds__(kBreadthPhaseThreads, 1)
-k_breadth_phases(mp_batch bt, int32_t policy, int64_t* __restrict__ offsets, int64_t* __restrict__ plan_peak,
-                 int32_t* __restrict__ status, bool deferred_only) {
-    for (int32_t b = (int32_t)blockIdx.x; b < bt.n_traces; b += (int32_t)gridDim.x) {
-        if (deferred_only && status[b] != kBDeferred) continue;
-        const TraceView tv = load_trace(bt, b, false);
-        bool done = false;
-        if (tv.st == MP_OK) {
-            phases::Out o = {};
-            o.offsets = offsets + tv.lo;
-            o.plan_peak = plan_peak + b;
-            o.status = status + b;
-            done = phases::plan<true, false>(bt, tv, policy, o);
+k_breadth_rest(mp_batch bt, int32_t policy, int64_t* __restrict__ offsets, int64_t* __restrict__ plan_peak,
+               int32_t* __restrict__ status, unsigned char* __restrict__ ws, size_t ws_stride, bool deferred_only,
+               bool in_phases, bool by_tensor) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
+    // this CTA's traces are blockIdx.x + k * gridDim.x; their statuses are
+    // read 32 at a time by one warp
+    __shared__ unsigned s_todo;
+    for (int64_t k0 = 0; blockIdx.x + k0 * gridDim.x < bt.n_traces; k0 += 32) {
+        if (threadIdx.x < 32) {
+            const int64_t b = blockIdx.x + (k0 + threadIdx.x) * gridDim.x;
+            const unsigned m =
+                __ballot_sync(0xffffffffu, b < bt.n_traces && (!deferred_only || status[b] == kBDeferred));
+            if (threadIdx.x == 0) s_todo = m;
         }
-        if (!done && !deferred_only && threadIdx.x == 0) status[b] = kBDeferred;
         __syncthreads();
+        unsigned m = s_todo;
+        __syncthreads();
+        for (; m; m &= m - 1) {
+            const int b = (int)(blockIdx.x + (k0 + __ffs(m) - 1) * gridDim.x);
+            bool done = false;
+            if (in_phases) {
+                const TraceView tv = load_trace(bt, b, false);
+                if (tv.st == MP_OK) {
+                    phases::Out o = {};
+                    o.offsets = offsets + tv.lo;
+                    o.plan_peak = plan_peak + b;
+                    o.status = status + b;
+                    done = phases::plan<true, false>(bt, tv, policy, o);
+                }
+            }
+            if (!done && by_tensor) breadth_trace<kSmem>(b, bt, policy, offsets, plan_peak, status, ws, ws_stride);
+            if (!done && !by_tensor && threadIdx.x == 0) status[b] = kBDeferred;  // left to the next launch
+            __syncthreads();
+        }
     }
 }
 
 bool breadth_comp_fits(const mp_batch& bt) {
     return BCompLayout(bt.max_tensors, bt.max_steps).total <= kSmemCeiling;
+}
+
+// One launch of k_breadth_rest: in phases, tensor by tensor, or both.
+template <bool kSmem>
+cudaError_t launch_rest_once(const mp_batch& bt, int32_t policy, int64_t* offsets, int64_t* plan_peak, int32_t* status,
+                             void* workspace, bool deferred_only, bool in_phases, bool by_tensor,
+                             cudaStream_t stream) {
+    const size_t data = BreadthLayout(bt.max_tensors, bt.max_steps).total;
+    size_t smem = kSmem && by_tensor ? data : 0;
+    if (in_phases) smem = std::max(smem, phases::smem_bytes<true>(bt));
+    const void* fn = (const void*)k_breadth_rest<kSmem>;
+    int sms = 0, resident = 0;
+    cudaError_t e = sm_count(&sms);
+    // more traces than SMs: half the threads, so that an SM holds two
+    const int threads = bt.n_traces > sms ? kBreadthPhaseThreads / 2 : kBreadthPhaseThreads;
+    if (e == cudaSuccess) e = set_smem_limit(fn, smem);
+    if (e == cudaSuccess) e = max_resident_ctas(fn, threads, smem, &resident);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)std::min(bt.n_traces, resident));
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = deferred_only ? 1 : 0;  // (it follows a kernel of this call)
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_breadth_rest<kSmem>, bt, policy, offsets, plan_peak, status,
+                              static_cast<unsigned char*>(workspace), data, deferred_only, in_phases, by_tensor);
+}
+
+// Both ways in one launch where that leaves room for two CTAs an SM, else one
+// launch each: 256 traces of 2,000 tensors take 0.32 ms so, and 0.45 ms with
+// the 160 KB that placing one of them tensor by tensor would need.
+template <bool kSmem>
+cudaError_t launch_rest(const mp_batch& bt, int32_t policy, int64_t* offsets, int64_t* plan_peak, int32_t* status,
+                        void* workspace, bool deferred_only, bool in_phases, cudaStream_t stream) {
+    const size_t data = BreadthLayout(bt.max_tensors, bt.max_steps).total;
+    if (kSmem && in_phases && data > std::max(phases::smem_bytes<true>(bt), kTwoPerSm)) {
+        const cudaError_t e = launch_rest_once<kSmem>(bt, policy, offsets, plan_peak, status, workspace, deferred_only,
+                                                      true, false, stream);
+        if (e != cudaSuccess) return e;
+        return launch_rest_once<kSmem>(bt, policy, offsets, plan_peak, status, workspace, true, false, true, stream);
+    }
+    return launch_rest_once<kSmem>(bt, policy, offsets, plan_peak, status, workspace, deferred_only, in_phases, true,
+                                   stream);
 }
 
 }  // namespace
@@ -789,33 +862,8 @@ cudaError_t launch_breadth(const mp_batch& bt, int32_t policy, int64_t* offsets,
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
-    if (in_phases && bt.max_tensors > kBWarpComp) {
-        // more traces than SMs: half the threads, so that an SM holds two
-        const size_t pbytes = phases::smem_bytes<true>(bt);
-        const void* fn = (const void*)k_breadth_phases;
-        int sms = 0, resident = 0;
-        cudaError_t e = sm_count(&sms);
-        const int threads = bt.n_traces > sms ? kBreadthPhaseThreads / 2 : kBreadthPhaseThreads;
-        if (e == cudaSuccess) e = set_smem_limit(fn, pbytes);
-        if (e == cudaSuccess) e = max_resident_ctas(fn, threads, pbytes, &resident);
-        if (e != cudaSuccess) return e;
-        k_breadth_phases<<<(unsigned)std::min(bt.n_traces, resident), threads, pbytes, stream>>>(
-            bt, policy, offsets, plan_peak, status, comp);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-    }
-    const bool deferred_only = comp || (in_phases && bt.max_tensors > kBWarpComp);
-    const size_t bytes = BreadthLayout(bt.max_tensors, bt.max_steps).total;
-    if (breadth_fits_smem(bt)) {
-        cudaError_t e = set_smem_limit((const void*)k_breadth<true>, bytes);
-        if (e != cudaSuccess) return e;
-        k_breadth<true><<<(unsigned)bt.n_traces, kBreadthThreads, bytes, stream>>>(bt, policy, offsets, plan_peak,
-                                                                                   status, nullptr, 0, deferred_only);
-    } else {
-        k_breadth<false><<<(unsigned)bt.n_traces, kBreadthThreads, 0, stream>>>(
-            bt, policy, offsets, plan_peak, status, static_cast<unsigned char*>(workspace), bytes, deferred_only);
-    }
-    return cudaGetLastError();
+    return breadth_fits_smem(bt) ? launch_rest<true>(bt, policy, offsets, plan_peak, status, workspace, comp, in_phases, stream)
+                                 : launch_rest<false>(bt, policy, offsets, plan_peak, status, workspace, comp, in_phases, stream);
 }
 
 }  // namespace mp
