@@ -28,8 +28,8 @@
 //                  zero;
 //   k_grid_finish  a warp per 32 tensors: offsets back by tensor id, the plan
 //                  peak, and (fused) every lifetime-overlapping pair checked
-//                  for address overlap;
-//   k_grid_final   one thread per trace: peaks, verdicts, statuses.
+//                  for address overlap; the last CTA writes the traces' peaks,
+//                  verdicts and statuses.
 //
 // Candidates.  A short-lived tensor (life at most kGridLong steps) overlaps
 // tensor x only if it is allocated in (a_x - lw, f_x), lw being the longest
@@ -254,7 +254,7 @@ __device__ __forceinline__ void push(const GridWs& w, int64_t slot) {
     __threadfence();  // every predecessor's offset, and the class, before the queue entry
     const bool cta = __ldcg(w.cls + slot) != 0;
     const int32_t at = atomicAdd(cta ? &w.ctl->tail_l : &w.ctl->tail_s, 1);
-    st_rlx((cta ? w.ql : w.qs) + at, (int32_t)slot);
+    st_rlx((cta ? w.ql : w.qs) + at, (int32_t)slot + 1);
 }
 
 // ---------------------------------------------------------------- prep
@@ -1024,7 +1024,7 @@ __device__ int32_t take_slot(const GridWs& w, const int32_t* queue, const int32_
     int32_t seen = -1, dist = 0;
     for (int32_t polls = 0;; ++polls) {
         const int32_t v = ld_rlx(queue + h);
-        if (v >= 0) return v;
+        if (v > 0) return v - 1;
         if ((polls & 7) == 0) {
             if (ld_rlx(&ctl->fail)) return -1;
             const int32_t placed = ld_rlx(&ctl->placed);
@@ -1209,14 +1209,40 @@ __global__ void __launch_bounds__(kFarThreads, 1) k_grid_phases(mp_batch bt, int
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ phases::Shared sh;
     __shared__ FarShared fs;
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // for the flow kernel
+    asm volatile("griddepcontrol.launch_dependents;");
     const TraceInfo* ti = w.ti + blockIdx.x;
     if (ti->ok && in_phases(w.ctl) && w.ctl->fail == 0) far_place(w, (int32_t)blockIdx.x, policy, smem_raw, sh, fs);
 }
 
 // ---------------------------------------------------------------- finish
 
+// Peaks, verdicts and statuses, a thread per trace.
+template <bool kFused>
+__device__ __forceinline__ void grid_final(const mp_batch& bt, const GridOut& out, const GridWs& w) {
+    for (int64_t b = threadIdx.x; b < bt.n_traces; b += blockDim.x) {
+        TraceInfo* tp = w.ti + b;
+        TraceInfo ti = *tp;
+        ti.peak = __ldcg(&tp->peak);  // (written by other CTAs' atomics)
+        ti.key = __ldcg(&tp->key);
+        ti.incomplete = __ldcg(&tp->incomplete);
+        if (!ti.ok) continue;  // its status was written by the prep kernel
+        out.plan_peak[b] = (int64_t)ti.peak;
+        out.status[b] = ti.incomplete ? MP_ETIMEOUT : MP_OK;
+        if (kFused) {
+            const bool good = ti.key == ~0ull;
+            if (out.verdict) out.verdict[b] = good ? 1 : 0;
+            if (out.conflict) {
+                out.conflict[2 * b] = good ? -1 : (int32_t)(ti.key >> 32);
+                out.conflict[2 * b + 1] = good ? -1 : (int32_t)(ti.key & 0xffffffffu);
+            }
+        }
+    }
+}
+
 template <bool kFused>
 __global__ void __launch_bounds__(kFinishThreads) k_grid_finish(mp_batch bt, GridOut out, GridWs w) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // for the kernel that placed the last tensors
     const int lane = threadIdx.x & 31;
     const unsigned full = 0xffffffffu;
     const int64_t M = w.M;
@@ -1291,23 +1317,15 @@ __global__ void __launch_bounds__(kFinishThreads) k_grid_finish(mp_batch bt, Gri
             }
         }
     }
-}
-
-template <bool kFused>
-__global__ void k_grid_final(mp_batch bt, GridOut out, GridWs w) {
-    const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= bt.n_traces) return;
-    const TraceInfo ti = w.ti[b];
-    if (!ti.ok) return;  // its status was written by the prep kernel
-    out.plan_peak[b] = (int64_t)ti.peak;
-    out.status[b] = ti.incomplete ? MP_ETIMEOUT : MP_OK;
-    if (kFused) {
-        const bool good = ti.key == ~0ull;
-        if (out.verdict) out.verdict[b] = good ? 1 : 0;
-        if (out.conflict) {
-            out.conflict[2 * b] = good ? -1 : (int32_t)(ti.key >> 32);
-            out.conflict[2 * b + 1] = good ? -1 : (int32_t)(ti.key & 0xffffffffu);
-        }
+    // the last CTA to get here sees every other's results and sums them up
+    __shared__ bool s_last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(&w.ctl->finished, 1) == (int32_t)gridDim.x - 1;
+    __syncthreads();
+    if (s_last) {
+        __threadfence();
+        grid_final<kFused>(bt, out, w);
     }
 }
 
@@ -1336,7 +1354,9 @@ GridLayout grid_layout(const mp_batch& bt) {
         at = bytes > SIZE_MAX - kAlign ? SIZE_MAX : add_sat(at, align_up(bytes));
         return here;
     };
-    L.ctl = take(sizeof(GridCtl));
+    L.ctl = take(sizeof(GridCtl));  // the control block and the queues, cleared together
+    L.qs = take(mul_sat(slots, 4));
+    L.ql = take(mul_sat(slots, 4));
     L.ti = take(mul_sat(B, sizeof(TraceInfo)));
     L.bend = take(mul_sat(mul_sat(B, TS), 4));
     L.rec = take(mul_sat(slots, sizeof(GRec)));
@@ -1344,8 +1364,6 @@ GridLayout grid_layout(const mp_batch& bt) {
     L.off = take(mul_sat(slots, 8));
     L.cnt = take(mul_sat(slots, 4));
     L.cls = take(mul_sat(slots, 4));
-    L.qs = take(mul_sat(slots, 4));
-    L.ql = take(mul_sat(slots, 4));
     L.ll = take(mul_sat(slots, 4));
     // a long-lived tensor has fewer than max_tensors predecessors; BEST sorts a
     // power of two of pairs
@@ -1405,6 +1423,24 @@ GridWs grid_ws(const mp_batch& bt, const GridLayout& L, unsigned char* ws) {
     return w;
 }
 
+// Launches a kernel that waits for the previous one's grid itself, so that its
+// launch overlaps that grid's end.
+template <typename... Params, typename... Args>
+cudaError_t launch_after(void (*kernel)(Params...), unsigned grid, unsigned threads, size_t smem, cudaStream_t stream,
+                         Args&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 template <bool kFused>
 cudaError_t launch_grid_impl(const mp_batch& bt, const GridOut& out, void* workspace, int32_t hold,
                              cudaStream_t stream) {
@@ -1413,8 +1449,7 @@ cudaError_t launch_grid_impl(const mp_batch& bt, const GridOut& out, void* works
     unsigned char* ws = static_cast<unsigned char*>(workspace);
     GridWs w = grid_ws(bt, L, ws);
     w.hold = hold;
-    cudaError_t e = cudaMemsetAsync(ws + L.ctl, 0, sizeof(GridCtl), stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(ws + L.qs, 0xff, L.ll - L.qs, stream);  // both queues: -1
+    cudaError_t e = cudaMemsetAsync(ws + L.ctl, 0, L.ti - L.ctl, stream);
     if (e != cudaSuccess) return e;
     k_grid_prep<kFused><<<(unsigned)bt.n_traces, kPrepThreads, 0, stream>>>(bt, out, w);
     e = cudaGetLastError();
@@ -1439,8 +1474,7 @@ cudaError_t launch_grid_impl(const mp_batch& bt, const GridOut& out, void* works
     if (L.phased && hold < 0) {
         e = set_smem_limit((const void*)k_grid_phases, kFarSmem);
         if (e != cudaSuccess) return e;
-        k_grid_phases<<<(unsigned)bt.n_traces, kFarThreads, kFarSmem, stream>>>(bt, policy, w);
-        e = cudaGetLastError();
+        e = launch_after(k_grid_phases, (unsigned)bt.n_traces, kFarThreads, kFarSmem, stream, bt, policy, w);
         if (e != cudaSuccess) return e;
     }
 
@@ -1451,11 +1485,8 @@ cudaError_t launch_grid_impl(const mp_batch& bt, const GridOut& out, void* works
     const int64_t warps_needed = ((int64_t)bt.n_traces * w.M + 31) / 32;
     const int64_t blocks = std::min<int64_t>((warps_needed + (kFinishThreads / 32) - 1) / (kFinishThreads / 32),
                                              (int64_t)sms * 8);
-    k_grid_finish<kFused><<<(unsigned)std::max<int64_t>(blocks, 1), kFinishThreads, 0, stream>>>(bt, out, w);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_grid_final<kFused><<<(unsigned)((bt.n_traces + 255) / 256), 256, 0, stream>>>(bt, out, w);
-    return cudaGetLastError();
+    return launch_after(k_grid_finish<kFused>, (unsigned)std::max<int64_t>(blocks, 1), kFinishThreads, 0, stream, bt,
+                        out, w);
 }
 
 }  // namespace

@@ -80,7 +80,7 @@ struct GridCtl {
     int32_t checked;         // traces that passed their checks ...
     int32_t votes, neutral;  // ... for which phases pay, and which fit them (choose_phases)
     int32_t arrived;         // CTAs that reached the grid's barriers, all told
-    int32_t pad;
+    int32_t finished;        // CTAs of k_grid_finish that are done
 };
 
 // Whether the batch's traces are placed by one CTA each in phases
@@ -116,7 +116,7 @@ struct GridWs {
     int64_t* off;    // offset of each record (-1 until placed)
     int32_t* cnt;    // signed predecessor counts
     int32_t* cls;    // 1: a CTA item (long-lived, or more predecessors than a warp's buffer)
-    int32_t* qs;     // queue of ready warp items (slot ids, -1 = not filled)
+    int32_t* qs;     // queue of ready warp items (1 + slot id, 0 = not filled)
     int32_t* ql;     // queue of ready CTA items
     int32_t* ll;     // [B][max_tensors]: positions of the long-lived records, ascending
     int64_t* ovf;    // per long-capable CTA: pairs beyond the shared region
