@@ -211,22 +211,39 @@ __device__ __forceinline__ void block_min_pair(int64_t& key, int64_t& val, int64
 }
 
 // Exclusive scan of per-thread values over the block; returns this thread's
-// prefix and writes the block total to *total.
+// prefix and writes the block total to *total.  One barrier: every warp sums
+// the warp totals for itself, instead of one warp doing it between two more
+// (the fused pass over 4,096 traces of 512 tensors: 110.1 us so, 108.4 with one
+// barrier a scan).  It does not end with one: red may be written again only
+// after the caller's next barrier.
 template <typename V>
-__device__ __forceinline__ V block_excl_scan(V v, V* red, V* total) {
+__device__ __forceinline__ V block_excl_scan_open(V v, V* red, V* total) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-    V incl = warp_incl_scan(v);
+    const V incl = warp_incl_scan(v);
     if (lane == 31) red[w] = incl;
     __syncthreads();
-    if (w == 0) {
-        V x = lane < nw ? red[lane] : V(0);
-        V xs = warp_incl_scan(x);
-        if (lane < nw) red[lane] = xs - x;  // exclusive prefix of warp totals
-        if (lane == nw - 1) red[32] = xs;
+    V before = 0, sum = 0;
+    if (nw <= 4) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const V x = k < nw ? red[k] : V(0);
+            before += k < w ? x : V(0);
+            sum += x;
+        }
+    } else {
+        const V x = lane < nw ? red[lane] : V(0);
+        const V xs = warp_incl_scan(x);
+        sum = __shfl_sync(0xffffffffu, xs, 31);
+        before = __shfl_sync(0xffffffffu, xs - x, w);
     }
-    __syncthreads();
-    V r = red[w] + incl - v;
-    *total = red[32];
+    *total = sum;
+    return before + incl - v;
+}
+
+// The same with a barrier at its end.
+template <typename V>
+__device__ __forceinline__ V block_excl_scan(V v, V* red, V* total) {
+    const V r = block_excl_scan_open(v, red, total);
     __syncthreads();
     return r;
 }
@@ -248,7 +265,7 @@ __device__ V block_excl_scan_array(V* x, int64_t len, V* red) {
             sum += loc[k];
         }
         V tot;
-        V pre = block_excl_scan<V>(sum, red, &tot) + carry;
+        V pre = block_excl_scan_open<V>(sum, red, &tot) + carry;
 #pragma unroll
         for (int k = 0; k < ITEMS; ++k) {
             if (my + k < len) x[my + k] = pre;
@@ -289,6 +306,46 @@ __device__ int64_t block_incl_scan_max_i64(int64_t* x, int64_t len, int64_t init
         __syncthreads();
     }
     return block_max_i64(mx, red);
+}
+
+// Writes a warp's 256 consecutive profile values (8 per lane) to global memory:
+// base is the warp's first step, at(t) the shared-memory word of step t, v the
+// lane's steps base + 8 lane .. + 7.  Each lane's 8 words go back to shared
+// memory and leave it two steps a lane, so that a warp's store covers 512
+// consecutive bytes; stored straight from registers, 16 bytes every 64, each
+// store touches four times as many cache lines (live profiles of 4,096 traces of
+// 1,024 steps: 20.5 us so, 18.4 this way).
+template <typename W, typename At>
+__device__ __forceinline__ void warp_store_profile(int64_t* __restrict__ out, int32_t base, int32_t T, bool vec,
+                                                   const W (&v)[8], At&& at) {
+    const int32_t lane = (int32_t)(threadIdx.x & 31), my = base + 8 * lane;
+    if (my + 8 <= T) {
+        W* run = at(my);  // 16-byte aligned, the 8 words consecutive
+        if constexpr (sizeof(W) == 8) {
+#pragma unroll
+            for (int k = 0; k < 8; k += 2)
+                *reinterpret_cast<longlong2*>(run + k) = make_longlong2((int64_t)v[k], (int64_t)v[k + 1]);
+        } else {
+            *reinterpret_cast<uint4*>(run) = make_uint4(v[0], v[1], v[2], v[3]);
+            *reinterpret_cast<uint4*>(run + 4) = make_uint4(v[4], v[5], v[6], v[7]);
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+            if (my + k < T) *at(my + k) = v[k];
+    }
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const int32_t t = base + 64 * r + 2 * lane;
+        if (t + 1 < T && vec) {
+            const W* p = at(t);
+            *reinterpret_cast<longlong2*>(out + t) = make_longlong2((int64_t)p[0], (int64_t)p[1]);
+        } else {
+            if (t < T) out[t] = (int64_t)*at(t);
+            if (t + 1 < T) out[t + 1] = (int64_t)*at(t + 1);
+        }
+    }
 }
 
 }  // namespace mp

@@ -1152,7 +1152,7 @@ __device__ __forceinline__ void d_add(uint32_t* d, int64_t v) { atomicAdd(d, (ui
 // wrap: every prefix of a trace's profile is below 2^32 on the 32-bit path).
 template <typename W>
 __device__ __forceinline__ W block_excl_scan_w(W v, int64_t* red, W* total) {
-    return block_excl_scan<W>(v, reinterpret_cast<W*>(red), total);
+    return block_excl_scan_open<W>(v, reinterpret_cast<W*>(red), total);
 }
 
 // Components of more than kWalkMin members without long-lived ones are walked
@@ -1573,6 +1573,7 @@ __device__ __forceinline__ void plan_trace(const int b, const mp_batch& bt, cons
         for (int32_t base_t = 0; base_t < T; base_t += (int32_t)blockDim.x * kRun) {
             const int32_t my = base_t + (int32_t)threadIdx.x * kRun;
             const W* run = D + dpos<W>(my);
+            if (base_t > 0) __syncthreads();  // red: the previous tile's totals are read
             W v[kRun];
             if (my + kRun <= T) {
 #pragma unroll
@@ -1602,7 +1603,11 @@ __device__ __forceinline__ void plan_trace(const int b, const mp_batch& bt, cons
                 v[k] += pre;
                 lmax = v[k] > lmax ? v[k] : lmax;
             }
-            if (vec_out && my + kRun <= T) {
+            if constexpr (kSmem) {
+                // (a warp only rewrites words that it alone has read)
+                warp_store_profile<W>(pout, base_t + (int32_t)(threadIdx.x & ~31u) * kRun, T, vec_out, v,
+                                      [&](int32_t t) { return D + dpos<W>(t); });
+            } else if (vec_out && my + kRun <= T) {
 #pragma unroll
                 for (int k = 0; k < kRun; k += 2)
                     *reinterpret_cast<longlong2*>(pout + my + k) = make_longlong2((int64_t)v[k], (int64_t)v[k + 1]);

@@ -67,6 +67,7 @@ __device__ __forceinline__ int64_t scan_and_write(W* D, int64_t* out, int32_t T,
         const int32_t my = base + tid * kProfItems;
         W v[kProfItems];
         const W* run = D + dpos<kSmem, W>(my);
+        if (base > 0) __syncthreads();  // red: the previous tile's totals are read
         if (vec_d && my + kProfItems <= T) {
 #pragma unroll
             for (int k = 0; k < kProfItems; k += kVec) {
@@ -89,14 +90,18 @@ __device__ __forceinline__ int64_t scan_and_write(W* D, int64_t* out, int32_t T,
 #pragma unroll
         for (int k = 1; k < kProfItems; ++k) v[k] += v[k - 1];
         W tot;
-        const W pre = block_excl_scan<W>(v[kProfItems - 1], reinterpret_cast<W*>(red), &tot) + carry;
+        const W pre = block_excl_scan_open<W>(v[kProfItems - 1], reinterpret_cast<W*>(red), &tot) + carry;
         carry += tot;
 #pragma unroll
         for (int k = 0; k < kProfItems; ++k) {
             v[k] += pre;
             mx = v[k] > mx ? v[k] : mx;
         }
-        if (vec_out && my + kProfItems <= T) {
+        if constexpr (kSmem) {
+            // (a warp only rewrites words that it alone has read)
+            warp_store_profile<W>(out, base + (tid & ~31) * kProfItems, T, vec_out, v,
+                                  [&](int32_t t) { return D + dpos<kSmem, W>(t); });
+        } else if (vec_out && my + kProfItems <= T) {
 #pragma unroll
             for (int k = 0; k < kProfItems; k += 2)
                 *reinterpret_cast<longlong2*>(out + my + k) = make_longlong2((int64_t)v[k], (int64_t)v[k + 1]);

@@ -90,7 +90,8 @@ __device__ void block_excl_scan_i32(int32_t* x, int32_t len, int32_t* red) {
 #pragma unroll
         for (int k = 0; k < kValItems; ++k) sum += v[k];
         int32_t tot;
-        int32_t pre = block_excl_scan<int32_t>(sum, red, &tot) + carry;
+        if (base > 0) __syncthreads();  // red: the previous tile's totals are read
+        int32_t pre = block_excl_scan_open<int32_t>(sum, red, &tot) + carry;
 #pragma unroll
         for (int k = 0; k < kValItems; ++k) {
             const int32_t t = v[k];
