@@ -14,7 +14,6 @@ constexpr int kProfileThreads = 128;  // one CTA per trace
 constexpr int kValidateThreads = 128;
 constexpr int kPeakThreads = 128;
 constexpr int kBumpThreads = 128;
-constexpr int kOptThreads = 128;
 constexpr int kReplayThreads = 256;
 constexpr int kBreadthThreads = 128;
 constexpr int kBreadthPhaseThreads = 512;  // half of it when the batch has more traces than the GPU SMs
@@ -87,7 +86,7 @@ cudaError_t launch_peak(const mp_batch& bt, const int64_t* offsets, int64_t* pla
 
 // Batches of at most kGridMaxTraces traces whose max_tensors exceeds
 // kGridMinTensors -- a few large traces -- are planned by the
-// grid-wide planners (grid.cu, grid_phases.cu); every other batch by one CTA
+// grid-wide planners (grid.cu, grid_phases.cuh); every other batch by one CTA
 // per trace (plan.cuh).
 constexpr int32_t kGridMinTensors = 1024;
 constexpr int32_t kGridMaxTraces = 32;

@@ -30,8 +30,10 @@
 //     stands as (larger id, smaller id) has an equal, earlier one;
 //   - the heaviest step's live bytes bound every plan from below: once an order
 //     reaches them, no later one can win.
-// 4,096 traces of 9 tensors over 6 steps: placing all 9! orders took 184 ms,
-// this search takes 3.7 ms.
+// A prefix dropped by its first tensors alone takes every later prefix that
+// starts with them along.  4,096 traces of 9 tensors over 6 steps: placing all 9!
+// orders took 184 ms, this search takes 1.8 ms, bound by the few traces with
+// over 10,000 nodes.
 //
 // Bytes are counted in units of the largest power of two that divides every
 // size of the trace: every offset is a sum of sizes, so nothing is rounded,
@@ -45,12 +47,11 @@ namespace mp {
 namespace {
 
 constexpr int kOptMax = 10;
-constexpr int kOptDepth = 2;  // tensors of a prefix: at most 90 subtrees of at most 8! orders a trace
-constexpr int kOptWarps = kOptThreads / 32;
+constexpr int kOptDepth = 3;  // tensors of a prefix: at most 720 subtrees of at most 7! orders a trace
 
 // The workspace that the entry point asks its callers for: 16 bytes per
 // kOptChunk orders of a trace.  The search itself needs none.
-constexpr int64_t kOptChunk = (int64_t)kOptThreads * 32;
+constexpr int64_t kOptChunk = 4096;
 
 __host__ __device__ constexpr int64_t factorial(int n) { return n <= 1 ? 1 : n * factorial(n - 1); }
 
@@ -178,6 +179,12 @@ struct Search {
         return __any_sync(kFull, (lane < n && hopeless(bound, q, b)) || (open && hopeless((W)(fit + size), q, b)));
     }
 
+    // The prefixes of q's block (of the given size) are done with.
+    __device__ bool skip(uint32_t q, uint32_t block) {
+        if (lane == 0) atomicMax(&sh.task, (q / block + 1) * block);
+        return true;
+    }
+
     // Walks the orders of prefix q; returns whether later prefixes matter.
     __device__ bool subtree(uint32_t q, int depth) {
         const uint32_t full = (1u << n) - 1u;
@@ -192,8 +199,10 @@ struct Search {
             rank %= below;
             const int j = __ffs(ids) - 1;
             const int prev = d ? nib(perm, d - 1) : -1;
-            if (prev > j && !((__shfl_sync(kFull, ov, j) >> prev) & 1u)) return true;
-            if (dead(q, fit)) return true;
+            // a prefix that leads nowhere takes all later ones with the same
+            // first tensors with it
+            if (prev > j && !((__shfl_sync(kFull, ov, j) >> prev) & 1u)) return skip(q, below);
+            if (dead(q, fit)) return skip(q, below * (uint32_t)(n - d));
             const W o = __shfl_sync(kFull, fit, j), e = o + __shfl_sync(kFull, size, j);
             peak = e > peak ? e : peak;
             place(j, o);
@@ -306,11 +315,12 @@ __device__ int64_t search_trace(OptShared& sh, W (*fits)[32], int n, int shift, 
     return (int64_t)opt << shift;
 }
 
-__global__ void __launch_bounds__(kOptThreads)
+template <int kThreads>
+__global__ void __launch_bounds__(kThreads)
 k_opt_search(mp_batch bt, int64_t* __restrict__ offsets, int64_t* __restrict__ opt_peak,
              int32_t* __restrict__ status) {
     __shared__ OptShared sh;
-    __shared__ int64_t fits[kOptWarps][kOptMax][32];  // (32-bit words use half of it)
+    __shared__ int64_t fits[kThreads / 32][kOptMax][32];  // (32-bit words use half of it)
     const int b = blockIdx.x;
     const int tid = (int)threadIdx.x;
     const TraceView tv = load_trace(bt, b, false);
@@ -381,7 +391,15 @@ size_t optimal_workspace_bytes(const mp_batch& bt) {
 cudaError_t launch_optimal(const mp_batch& bt, int64_t* offsets, int64_t* opt_peak, int32_t* status,
                            cudaStream_t stream) {
     if (bt.n_traces == 0) return cudaSuccess;
-    k_opt_search<<<(unsigned)bt.n_traces, kOptThreads, 0, stream>>>(bt, offsets, opt_peak, status);
+    // The longer the traces, the longer the hardest of them holds the call up:
+    // more warps shorten it, fewer leave room for more traces.  4,096 traces
+    // with 128 / 256 / 512 threads: 6 tensors 85 / 124 / 226 us, 9 tensors 4.0 /
+    // 2.3 / 1.8 ms; 1,000 of 8 tensors 272 / 158 / 170 us.
+    const unsigned grid = (unsigned)bt.n_traces;
+    if (bt.max_tensors <= 4) k_opt_search<64><<<grid, 64, 0, stream>>>(bt, offsets, opt_peak, status);
+    else if (bt.max_tensors <= 6) k_opt_search<128><<<grid, 128, 0, stream>>>(bt, offsets, opt_peak, status);
+    else if (bt.max_tensors <= 8) k_opt_search<256><<<grid, 256, 0, stream>>>(bt, offsets, opt_peak, status);
+    else k_opt_search<512><<<grid, 512, 0, stream>>>(bt, offsets, opt_peak, status);
     return cudaGetLastError();
 }
 
