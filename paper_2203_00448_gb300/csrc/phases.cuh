@@ -47,7 +47,7 @@ constexpr uint32_t kLongestChain = 1024;  // positions a chain may span beside l
 constexpr int32_t kBatch = 512;        // tensors inserted into the sorted list at a time
 constexpr int32_t kHeads = 1024;       // chains of a run listed at a time
 constexpr int32_t kChunk = 16;         // sorted-list entries per thread: kMaxTensors / the fewest threads
-constexpr int32_t kNear = 32;          // neighbours listed per short tensor of a large trace (grid_phases.cu)
+constexpr int32_t kNear = 32;          // neighbours listed per short tensor of a large trace (grid_phases.cuh)
 constexpr int32_t kThreadChain = 8;    // chains up to this long within a run can be walked by one thread
 constexpr int32_t kTeamChain = 64;     // chains from this length on are walked by the whole CTA together ...
 constexpr int32_t kTeams = 4;          // ... up to this many of a run
@@ -255,7 +255,7 @@ __device__ void block_sort(uint64_t (&k)[E], uint64_t* buf) {
 
 // The trace being placed.  kFar: a large trace whose records by rank and
 // lifetimes are in global memory, with the neighbours of its short tensors
-// listed beforehand (grid_phases.cu).
+// listed beforehand (grid_phases.cuh).
 template <bool kFar>
 struct Ctx {
     uint2* oe;            // by position: (offset, end) in units; (0, 0) until placed
