@@ -1280,8 +1280,9 @@ static __device__ __noinline__ void sort_keys(int32_t n) {
 // out.profile is set), priority order (greedy_by_size, or greedy by breadth
 // with kBreadth), placement, validation (kCheck) and outputs.  Returns false,
 // with nothing but the profile written, when the trace is not one for this
-// path: an invalid tensor, sizes summing to 2^32 units or more, or too many
-// long tensors.
+// path: an invalid tensor, sizes summing to 2^32 units or more, too many long
+// tensors, or a long chain beside some.  Either way no thread touches the
+// dynamic shared memory any more when another one returns.
 template <bool kBreadth, bool kCheck>
 __device__ __forceinline__ bool plan(const mp_batch& bt, const TraceView& tv, int32_t policy, const Out& out) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1561,6 +1562,9 @@ __device__ __forceinline__ bool plan(const mp_batch& bt, const TraceView& tv, in
         if (flag && at < (uint32_t)kMaxLong) LR[at] = (uint16_t)r;
         nl += (int32_t)tot;
     }
+    // every thread's ranks are written before the caller's general path takes
+    // the shared memory over
+    __syncthreads();
     if (nl > kMaxLong || (nl > 0 && sh.far > kLongestChain)) return false;
     for (int32_t p = t; p < n; p += nt) OE[p] = make_uint2(0, 0);
     __syncthreads();

@@ -90,6 +90,28 @@ def test_phases_limits(cuda_lib, case):
     _check(tg.from_arrays(traces))
 
 
+@pytest.mark.parametrize("kind", ("long", "chain"))
+def test_phases_refuse_late(cuda_lib, kind):
+    """Every trace of the batch is refused only once its long-lived tensors'
+    ranks are written, in the shared memory that the general path then clears:
+    too many of them, or a chain of over 1,024 positions beside some."""
+    rng = np.random.default_rng(len(kind))
+    traces = []
+    for k in range(40):
+        n = 1100 + 7 * k
+        if kind == "long":
+            T, a, f, s = _trace(rng, n, 1200, 0.0, 64, 1 << 10)
+            nl = 769 + k
+            a[-nl:] = rng.integers(0, 300, nl)
+            f[-nl:] = a[-nl:] + rng.integers(33, 800, nl)
+        else:
+            T, a, f, s = _trace(rng, n, 220, 0.02, 64, 1 << 10, life=20, full_span=True)
+        traces.append((T, a, f, s))
+    ts = tg.from_arrays(traces)
+    for _ in range(4):
+        _check(ts)
+
+
 def _far_trace(rng, n, T, kind):
     a = rng.integers(0, T, n)
     f = a + rng.integers(1, 6, n)
