@@ -422,6 +422,7 @@ __device__ __forceinline__ void far_place(const GridWs& w, int32_t b, int32_t po
                                           phases::Shared& sh, FarShared& fs) {
     const TraceInfo* ti = w.ti + b;
     const int32_t n = ti->n, nl = ti->nlong, t = (int32_t)threadIdx.x, nt = (int32_t)blockDim.x;
+    if (n == 0) return;  // an empty trace has no record to load ahead
     const int lane = t & 31, warp = t >> 5, nwarps = nt >> 5;
     const int64_t base = (int64_t)b * w.M;
     const FarLayout L(n, nl);

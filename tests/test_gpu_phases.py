@@ -139,7 +139,8 @@ def _far_trace(rng, n, T, kind):
 
 @pytest.mark.parametrize("kind,n", (("long-tail", 5000), ("long-tail", 20000), ("full-span", 6001), ("crowded-steps", 7000),
                                     ("wide-sums", 4500), ("short-only", 23000), ("short-only", 24000),
-                                    ("all-long", 4200), ("mixed", 9000), ("phased", 9000)))
+                                    ("all-long", 4200), ("mixed", 9000), ("phased", 9000),
+                                    ("empty-first", 6000)))
 def test_large_traces_in_phases(cuda_lib, kind, n):
     """One large trace per SM (batches of a few, past what one CTA prepares in
     its shared memory), and those left to the grid-wide dataflow."""
@@ -147,8 +148,11 @@ def test_large_traces_in_phases(cuda_lib, kind, n):
 
     rng = np.random.default_rng(n + len(kind))
     kinds = {"mixed": ("long-tail", "full-span", "wide-sums", "short-only"),
-             "phased": ("long-tail", "full-span", "long-tail")}.get(kind, (kind,))
+             "phased": ("long-tail", "full-span", "long-tail"), "empty-first": ("full-span",)}.get(kind, (kind,))
     traces = [_far_trace(rng, n, n // 2 + 100, k) for k in kinds]
+    if kind == "empty-first":  # no record of their own to load, and none before them
+        none = np.zeros(0, np.int64)
+        traces = [(10, none, none, none), (0, none, none, none)] + traces
     if kind in ("mixed", "phased"):
         traces += [(10, np.zeros(0, np.int64), np.zeros(0, np.int64), np.zeros(0, np.int64)),
                    (9, np.array([0, 3]), np.array([4, 2]), np.array([8, 8])),  # free <= alloc
