@@ -781,6 +781,7 @@ k_breadth_rest(mp_batch bt, int32_t policy, int64_t* __restrict__ offsets, int64
                     o.offsets = offsets + tv.lo;
                     o.plan_peak = plan_peak + b;
                     o.status = status + b;
+                    o.hold = phases::test_team_hold(b);
                     done = phases::plan<true, false>(bt, tv, policy, o);
                 }
             }
@@ -867,3 +868,21 @@ cudaError_t launch_breadth(const mp_batch& bt, int32_t policy, int64_t* offsets,
 }
 
 }  // namespace mp
+
+#ifdef MP_TEST_HOOKS
+// Test builds only: mp_plan_greedy_by_breadth, except that the member at
+// alloc-order position hold_pos of trace hold_trace is never placed if a team
+// of warps walks its chain, so that the team's bounded waits run out.
+extern "C" __attribute__((visibility("default"))) mp_status mp_test_breadth_team_hold(
+    const mp_batch* batch, mp_fit_policy policy, int64_t* offsets, int64_t* plan_peak, int32_t* trace_status,
+    void* workspace, size_t workspace_bytes, int32_t hold_trace, int32_t hold_pos, void* stream) {
+    if (batch == nullptr || workspace_bytes < mp::breadth_workspace_bytes(*batch)) return MP_EINVAL;
+    const int32_t none[2] = {-1, -1}, held[2] = {hold_trace, hold_pos};
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    cudaError_t e = cudaMemcpyToSymbol(mp::phases::g_test_team_hold, held, sizeof(held));
+    if (e == cudaSuccess) e = mp::launch_breadth(*batch, policy, offsets, plan_peak, trace_status, workspace, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    const cudaError_t e2 = cudaMemcpyToSymbol(mp::phases::g_test_team_hold, none, sizeof(none));
+    return e == cudaSuccess && e2 == cudaSuccess ? MP_OK : MP_ECUDA;
+}
+#endif

@@ -1049,16 +1049,24 @@ __device__ int32_t take_slot(const GridWs& w, const int32_t* queue, const int32_
     }
 }
 
+// Test builds (MP_TEST_HOOKS) can keep one CTA from arriving at the grid's
+// barriers, so that the others' bounded waits run out.
+#ifdef MP_TEST_HOOKS
+__device__ __forceinline__ bool test_absent(const GridWs& w) { return w.hold == kHoldBarrier && blockIdx.x == 0; }
+#else
+__device__ __forceinline__ bool test_absent(const GridWs&) { return false; }
+#endif
+
 // Barrier over the grid, whose CTAs are all resident (a cooperative launch):
 // `round` counts its uses from 1.  Every CTA arrives without waiting for
 // anything but this, so it opens as soon as the slowest is there; the wait is
 // bounded like a worker's (false, with the flag raised, when it runs out).
-__device__ __forceinline__ bool grid_barrier(GridCtl* ctl, int32_t round) {
+__device__ __forceinline__ bool grid_barrier(GridCtl* ctl, int32_t round, bool absent) {
     __shared__ int32_t s_open;
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
-        atomicAdd(&ctl->arrived, 1);
+        if (!absent) atomicAdd(&ctl->arrived, 1);
         const int32_t want = round * (int32_t)gridDim.x;
         const long long t0 = clock64();
         int32_t open = 1;
@@ -1102,7 +1110,7 @@ k_grid_flow(mp_batch bt, int32_t policy, GridWs w, int32_t long_ctas) {
     GridCtl* ctl = w.ctl;
     if (in_phases(ctl)) {
         int32_t rounds = 0;
-        far_prepare(bt, w, smem_raw, red, [&]() { return grid_barrier(ctl, ++rounds); });
+        far_prepare(bt, w, smem_raw, red, [&]() { return grid_barrier(ctl, ++rounds, test_absent(w)); });
         return;
     }
 

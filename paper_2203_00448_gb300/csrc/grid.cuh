@@ -123,7 +123,7 @@ struct GridWs {
     int64_t ovf_pairs;
     int32_t M;       // max_tensors: the slot stride of a trace
     int32_t TS;      // max_steps: the bucket stride of a trace
-    int64_t hold;    // test hook: the slot that is never queued (-1: none)
+    int64_t hold;    // test hook: the slot that is never queued, or kHoldBarrier (-1: none)
     // For traces placed in phases, by slot (stable: alloc step, then id), or
     // by rank: null if no trace of the batch can be.
     uint32_t* p_af;  // lifetime: alloc | free << 16

@@ -90,6 +90,7 @@ cudaError_t launch_peak(const mp_batch& bt, const int64_t* offsets, int64_t* pla
 // per trace (plan.cuh).
 constexpr int32_t kGridMinTensors = 1024;
 constexpr int32_t kGridMaxTraces = 32;
+constexpr int32_t kHoldBarrier = -2;  // a test's hold_slot: a CTA that never arrives at the grid's barriers
 bool grid_path(const mp_batch& bt);
 size_t grid_workspace_bytes(const mp_batch& bt);
 // hold >= 0 is a test hook: the tensor with that slot id (trace * max_tensors

@@ -51,7 +51,11 @@ constexpr int32_t kNear = 32;          // neighbours listed per short tensor of 
 constexpr int32_t kThreadChain = 8;    // chains up to this long within a run can be walked by one thread
 constexpr int32_t kTeamChain = 64;     // chains from this length on are walked by the whole CTA together ...
 constexpr int32_t kTeams = 4;          // ... up to this many of a run
-constexpr int32_t kTeamPolls = 1 << 20;  // bound of a wait there (some 50 ms)
+#ifdef MP_TEST_SPIN_CYCLES
+constexpr long long kTeamSpinCycles = MP_TEST_SPIN_CYCLES;  // test builds: a short bound
+#else
+constexpr long long kTeamSpinCycles = 1ll << 31;  // bound of a wait there in which no member is placed
+#endif
 constexpr int32_t kListRun = 64;       // runs from this length on list the gaps between the long tensors first
 constexpr int32_t kFewPending = 8;     // up to this many are inserted by comparison with every entry
 constexpr uint32_t kScanChain = 128;  // chains are linked member by member up to this many looks per thread, else by a sort
@@ -134,11 +138,24 @@ struct Shared {
     unsigned long long hi, lo, bits, best;
     uint32_t best32, lb, far;
     int32_t bad, lw, cnt, next, cnt1, next1, teams, fail;
+    int32_t placed;  // rank of the last member a team placed
+    int32_t hold;    // test builds: alloc-order position of a team's member that is never placed (-1: none)
     uint16_t team[kTeams];
     uint32_t last_free;
     uint32_t before[kFewPending];
     unsigned long long key;
 };
+
+// Test builds (MP_TEST_HOOKS) can keep one member of a team from being placed,
+// so that the others' bounded waits run out: {trace, alloc-order position}.
+#ifdef MP_TEST_HOOKS
+static __device__ int32_t g_test_team_hold[2] = {-1, -1};
+__device__ __forceinline__ int32_t test_team_hold(int b) { return b == g_test_team_hold[0] ? g_test_team_hold[1] : -1; }
+__device__ __forceinline__ bool test_held(const Shared& sh, int32_t pos) { return pos == sh.hold; }
+#else
+__device__ __forceinline__ int32_t test_team_hold(int) { return -1; }
+__device__ __forceinline__ bool test_held(const Shared&, int32_t) { return false; }
+#endif
 
 __device__ __forceinline__ uint32_t umax2(uint32_t a, uint32_t b) { return a > b ? a : b; }
 
@@ -640,6 +657,29 @@ __device__ __forceinline__ uint32_t walk_plain(const Ctx<false>& c, int32_t r, i
     }
 }
 
+// The bound of a team's waits: a second in which no member is placed.  (One
+// member may keep the others waiting for some ms by itself: one whose window is
+// thousands of positions wide goes through it once for every level it is
+// stacked above.)
+struct TeamWait {
+    long long since = 0;
+    int32_t placed = -1;  // (no rank: the first look always sees a change)
+    // Called by the whole warp between polls, `polls` counting from 0: whether
+    // to give up.
+    __device__ __forceinline__ bool over(Shared& sh, int32_t polls) {
+        if ((polls & 63) != 63) return false;
+        const int32_t p = *(volatile int32_t*)&sh.placed;
+        const long long now = clock64();
+        if (p != placed) {
+            placed = p;
+            since = now;
+        }
+        const bool out = *(volatile int32_t*)&sh.fail != 0 || now - since > kTeamSpinCycles;
+        if (out) *(volatile int32_t*)&sh.fail = 1;
+        return __any_sync(0xffffffffu, out);
+    }
+};
+
 // Walks the run's long chains (of the components of sh.team[0, teams), their
 // members among ranks [r0, r1)) with every warp of the CTA, no gap between long
 // tensors needing a look: the warps are dealt out to the chains, take their
@@ -647,11 +687,12 @@ __device__ __forceinline__ uint32_t walk_plain(const Ctx<false>& c, int32_t r, i
 // predecessors are placed (the offsets it needs are what it polls), and places
 // it.  The lowest unplaced member's predecessors are placed and its warp has
 // nothing earlier left to do, so every wait ends; it is bounded all the same
-// (sh.fail).  A chain of equal sizes is deep but not a single path: 262 and 112
+// (TeamWait, sh.fail).  A chain of equal sizes is deep but not a single path: 262 and 112
 // activations of a residual network, 172 K cycles by a warp each, 100 K this way.
 __device__ __forceinline__ uint32_t walk_teams(const Ctx<false>& c, int32_t teams, int32_t r0, int32_t r1,
                                                const Longs& lg, Shared& sh) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned full = 0xffffffffu;
     const int32_t nwarps = (int32_t)(blockDim.x >> 5) / teams;  // per chain
     const int32_t mine = min(warp / nwarps, teams);             // (warps left over take none)
     int32_t n = 0, first = 0, end = 0;
@@ -675,31 +716,34 @@ __device__ __forceinline__ uint32_t walk_teams(const Ctx<false>& c, int32_t team
         const int32_t r = c.list[i];
         const Rec rc = c.rec[r];
         const Win w = c.win[r];
+        TeamWait wait;
+        uint32_t top;
         if (w.wide) {  // no mask of its predecessors: every earlier member's turn first
-            for (int32_t x = first + lane; x < i; x += 32)
-                for (int32_t polls = 0; oe[c.rec[c.list[x]].pos] == 0; ++polls)
-                    if (polls > kTeamPolls || *(volatile int32_t*)&sh.fail) {
-                        sh.fail = 1;
-                        break;
-                    }
-            __syncwarp();
-            mx = umax2(mx, place_short(c, r, lg));
-            continue;
-        }
-        const bool pred = (c.mask[r] >> lane) & 1u;
-        const int32_t q = w.w0 + lane;
-        unsigned long long v = 0;
-        for (int32_t polls = 0;; ++polls) {
-            if (pred) v = oe[q];
-            if (!__any_sync(0xffffffffu, pred && v == 0)) break;
-            if (polls > kTeamPolls || *(volatile int32_t*)&sh.fail) {
-                if (lane == 0) sh.fail = 1;
-                break;
+            for (int32_t x0 = first; x0 < i; x0 += 32) {
+                const bool pred = x0 + lane < i;
+                const int32_t q = pred ? c.rec[c.list[x0 + lane]].pos : 0;
+                for (int32_t polls = 0; __any_sync(full, pred && oe[q] == 0); ++polls)
+                    if (wait.over(sh, polls)) break;
             }
+            __syncwarp();
+            if (test_held(sh, rc.pos)) continue;
+            top = place_short(c, r, lg);
+        } else {
+            const bool pred = (c.mask[r] >> lane) & 1u;
+            const int32_t q = w.w0 + lane;
+            unsigned long long v = 0;
+            for (int32_t polls = 0;; ++polls) {
+                if (pred) v = oe[q];
+                if (!__any_sync(full, pred && v == 0)) break;
+                if (wait.over(sh, polls)) break;
+            }
+            if (test_held(sh, rc.pos)) continue;
+            const uint32_t o = fit_plain(make_uint2((uint32_t)v, (uint32_t)(v >> 32)), rc.s, lg.top, c.policy);
+            top = o + rc.s;
+            if (lane == 0) oe[rc.pos] = ((unsigned long long)top << 32) | o;
         }
-        const uint32_t o = fit_plain(make_uint2((uint32_t)v, (uint32_t)(v >> 32)), rc.s, lg.top, c.policy);
-        if (lane == 0) oe[rc.pos] = ((unsigned long long)(o + rc.s) << 32) | o;
-        mx = umax2(mx, o + rc.s);
+        if (lane == 0) *(volatile int32_t*)&sh.placed = r;
+        mx = umax2(mx, top);
     }
     __syncthreads();
     return mx;
@@ -1239,6 +1283,7 @@ struct Out {
     int64_t* peak_lb;
     int32_t* verdict;
     int32_t* conflict;   // a pair
+    int32_t hold;        // test_team_hold of the trace
 };
 
 template <int E>
@@ -1313,6 +1358,8 @@ __device__ __forceinline__ bool plan(const mp_batch& bt, const TraceView& tv, in
         sh.bad = 0;
         sh.lw = 1;
         sh.fail = 0;
+        sh.placed = 0;
+        sh.hold = out.hold;
         sh.hi = sh.lo = sh.bits = 0;
         sh.lb = sh.far = sh.last_free = 0;
         sh.key = ~0ull;

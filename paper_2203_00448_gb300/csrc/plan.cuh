@@ -1890,6 +1890,7 @@ __device__ __forceinline__ bool plan_in_phases(const int b, const mp_batch& bt, 
     o.offsets = out.offsets + tv.lo;
     o.plan_peak = out.plan_peak + b;
     o.status = out.status + b;
+    o.hold = phases::test_team_hold(b);
     if (kFused) {
         if (out.profile) o.profile = out.profile + tv.plo;
         if (out.peak_lb) o.peak_lb = out.peak_lb + b;

@@ -7,9 +7,12 @@ trace then cannot finish: the workers waiting for that entry give up after the
 bound, the call returns, that trace reports MP_ETIMEOUT, the other traces of
 the batch are planned exactly as the oracle plans them, and the same library
 plans the same batch correctly right after (the context is still usable).
-Both waiting places are covered: the ready queue of the per-trace CTA tier
-(components with long-lived members), and the queues of the grid-wide planner
-(batches of a few traces of more than 1,024 tensors).
+The waiting places covered: the ready queue of the per-trace CTA tier
+(components with long-lived members), the queues of the grid-wide planner
+(batches of a few traces of more than 1,024 tensors), the barriers of its
+preparation for placement in phases (a CTA that never arrives; no trace of the
+batch can be placed then), and the teams of warps that walk a long chain of a
+trace placed in phases, by size and by breadth (a member that is never placed).
 """
 import ctypes
 
@@ -23,6 +26,7 @@ import tracegen as tg
 pytestmark = pytest.mark.gpu
 
 ETIMEOUT = 4
+HOLD_BARRIER = -2  # mp_test_plan_hold's hold_trace: a CTA that never arrives at the grid's barriers
 
 
 @pytest.fixture(scope="module")
@@ -31,24 +35,27 @@ def hooks_lib(cuda_lib):
 
     lib = ctypes.CDLL(build.build_test_hooks())
     P, BP = ctypes.c_void_p, ctypes.POINTER(_lib.MpBatch)
-    lib.mp_test_plan_hold.argtypes = [BP, ctypes.c_int32, P, P, P, P, ctypes.c_size_t, ctypes.c_int32,
-                                      ctypes.c_int32, P]
-    lib.mp_test_plan_hold.restype = ctypes.c_int32
+    for fn in (lib.mp_test_plan_hold, lib.mp_test_plan_team_hold, lib.mp_test_breadth_team_hold):
+        fn.argtypes = [BP, ctypes.c_int32, P, P, P, P, ctypes.c_size_t, ctypes.c_int32, ctypes.c_int32, P]
+        fn.restype = ctypes.c_int32
+    for fn in (lib.mp_plan_workspace_bytes, lib.mp_breadth_workspace_bytes):
+        fn.argtypes, fn.restype = [BP], ctypes.c_size_t
     return lib
 
 
-def _plan(lib, ts, policy, hold_trace, hold_pos):
+def _plan(lib, ts, policy, hold_trace, hold_pos, call="mp_test_plan_hold"):
     import paper_2203_00448_gb300 as mp
 
     db = mp.DeviceBatch.from_host(ts, "cuda")
-    need = mp.plan_workspace_bytes(db)
+    size = lib.mp_breadth_workspace_bytes if "breadth" in call else lib.mp_plan_workspace_bytes
+    need = size(ctypes.byref(db.struct()))
     ws = torch.empty(max(need, 256), dtype=torch.uint8, device="cuda")
     off = torch.full((ts.n_tensors,), -7, dtype=torch.int64, device="cuda")
     pk = torch.zeros(ts.n_traces, dtype=torch.int64, device="cuda")
     st = torch.full((ts.n_traces,), -7, dtype=torch.int32, device="cuda")
     s = db.struct()
-    rc = lib.mp_test_plan_hold(ctypes.byref(s), policy, off.data_ptr(), pk.data_ptr(), st.data_ptr(), ws.data_ptr(),
-                               ws.numel(), hold_trace, hold_pos, torch.cuda.current_stream().cuda_stream)
+    rc = getattr(lib, call)(ctypes.byref(s), policy, off.data_ptr(), pk.data_ptr(), st.data_ptr(), ws.data_ptr(),
+                            ws.numel(), hold_trace, hold_pos, torch.cuda.current_stream().cuda_stream)
     torch.cuda.synchronize()
     return rc, off.cpu().numpy(), pk.cpu().numpy(), st.cpu().numpy()
 
@@ -62,8 +69,8 @@ def _held_position(ts, b, alloc_step):
     return int((a < alloc_step).sum())
 
 
-def _check(ts, pol, off, pk, st, held):
-    o_off, o_pk, o_st = oracle.plan_greedy_by_size(ts, pol)
+def _check(ts, pol, off, pk, st, held, breadth=False):
+    o_off, o_pk, o_st = (oracle.plan_greedy_by_breadth if breadth else oracle.plan_greedy_by_size)(ts, pol)
     assert (o_st == 0).all()
     expect = np.zeros(ts.n_traces, dtype=np.int32)
     if held is not None:
@@ -133,3 +140,67 @@ def test_grid_wait_runs_out(hooks_lib, pol):
     rc, off, pk, st = _plan(hooks_lib, ts, pol, -1, -1)
     assert rc == mp.OK
     _check(ts, pol, off, pk, st, held=None)
+
+
+def _phased_grid_batch():
+    """Three traces of 1,500 tensors, 30 of which span the trace: placed in
+    phases by the grid-wide planner's rule."""
+    rng = np.random.default_rng(5)
+    traces = []
+    for _ in range(3):
+        n, T = 1500, 3000
+        a = rng.integers(0, T, n)
+        f = np.minimum(a + rng.integers(1, 6, size=n), T)
+        a[:30], f[:30] = 0, T
+        traces.append((T, a, f, rng.integers(1, 1 << 16, size=n) * 16))
+    return tg.from_arrays(traces)
+
+
+@pytest.mark.parametrize("pol", (oracle.FIT_FIRST, oracle.FIT_BEST))
+def test_grid_barrier_wait_runs_out(hooks_lib, pol):
+    import paper_2203_00448_gb300 as mp
+
+    ts = _phased_grid_batch()
+    rc, off, pk, st = _plan(hooks_lib, ts, pol, HOLD_BARRIER, 0)
+    assert rc == mp.OK
+    assert st.tolist() == [ETIMEOUT] * ts.n_traces
+    rc, off, pk, st = _plan(hooks_lib, ts, pol, -1, -1)  # nothing held
+    assert rc == mp.OK
+    _check(ts, pol, off, pk, st, held=None)
+
+
+def _team_batch(wide):
+    """36 traces, two of which are one chain: 400 tensors of few sizes, each
+    overlapping the next, walked by a team of warps; the one at position 200 is
+    the largest, so that its neighbours wait for it.  wide: behind the chain 300
+    small ones that are all alive together, whose windows are past a mask's 32
+    positions."""
+    rng = np.random.default_rng(6)
+    traces = []
+    for k in range(36):
+        n = 400 if k in (1, 20) else 50
+        a = np.arange(n)
+        f = a + rng.integers(2, 4, size=n)
+        s = rng.choice([1 << 20, 1 << 21], size=n)
+        s[n // 2] = 1 << 22
+        if wide and n == 400:
+            a = np.concatenate([a, np.full(300, n)])
+            f = np.concatenate([f, n + rng.integers(1, 4, size=300)])
+            s = np.concatenate([s, rng.choice([64, 128], size=300)])
+        traces.append((n + 10, a, f, s))
+    return tg.from_arrays(traces)
+
+
+@pytest.mark.parametrize("pol", (oracle.FIT_FIRST, oracle.FIT_BEST))
+@pytest.mark.parametrize("wide", (False, True))
+@pytest.mark.parametrize("call", ("mp_test_plan_team_hold", "mp_test_breadth_team_hold"))
+def test_team_wait_runs_out(hooks_lib, call, wide, pol):
+    import paper_2203_00448_gb300 as mp
+
+    ts, breadth = _team_batch(wide), "breadth" in call
+    rc, off, pk, st = _plan(hooks_lib, ts, pol, 1, 200, call)
+    assert rc == mp.OK
+    _check(ts, pol, off, pk, st, held=1, breadth=breadth)
+    rc, off, pk, st = _plan(hooks_lib, ts, pol, -1, -1, call)  # nothing held
+    assert rc == mp.OK
+    _check(ts, pol, off, pk, st, held=None, breadth=breadth)
