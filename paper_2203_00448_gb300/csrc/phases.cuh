@@ -52,9 +52,9 @@ constexpr int32_t kThreadChain = 8;    // chains up to this long within a run ca
 constexpr int32_t kTeamChain = 64;     // chains from this length on are walked by the whole CTA together ...
 constexpr int32_t kTeams = 4;          // ... up to this many of a run
 #ifdef MP_TEST_SPIN_CYCLES
-constexpr long long kTeamSpinCycles = MP_TEST_SPIN_CYCLES;  // test builds: a short bound
+constexpr int32_t kTeamPolls = 1 << 17;  // test builds: some 6 ms
 #else
-constexpr long long kTeamSpinCycles = 1ll << 31;  // bound of a wait there in which no member is placed
+constexpr int32_t kTeamPolls = 1 << 20;  // polls of a wait there (some 50 ms) in which some member has to be placed
 #endif
 constexpr int32_t kListRun = 64;       // runs from this length on list the gaps between the long tensors first
 constexpr int32_t kFewPending = 8;     // up to this many are inserted by comparison with every entry
@@ -138,7 +138,7 @@ struct Shared {
     unsigned long long hi, lo, bits, best;
     uint32_t best32, lb, far;
     int32_t bad, lw, cnt, next, cnt1, next1, teams, fail;
-    int32_t placed;  // rank of the last member a team placed
+    int32_t seen[16];  // by warp: members of its team placed when it last asked
     int32_t hold;    // test builds: alloc-order position of a team's member that is never placed (-1: none)
     uint16_t team[kTeams];
     uint32_t last_free;
@@ -657,38 +657,19 @@ __device__ __forceinline__ uint32_t walk_plain(const Ctx<false>& c, int32_t r, i
     }
 }
 
-// The bound of a team's waits: a second in which no member is placed.  (One
-// member may keep the others waiting for some ms by itself: one whose window is
-// thousands of positions wide goes through it once for every level it is
-// stacked above.)
-struct TeamWait {
-    long long since = 0;
-    int32_t placed = -1;  // (no rank: the first look always sees a change)
-    // Called by the whole warp between polls, `polls` counting from 0: whether
-    // to give up.
-    __device__ __forceinline__ bool over(Shared& sh, int32_t polls) {
-        if ((polls & 63) != 63) return false;
-        const int32_t p = *(volatile int32_t*)&sh.placed;
-        const long long now = clock64();
-        if (p != placed) {
-            placed = p;
-            since = now;
-        }
-        const bool out = *(volatile int32_t*)&sh.fail != 0 || now - since > kTeamSpinCycles;
-        if (out) *(volatile int32_t*)&sh.fail = 1;
-        return __any_sync(0xffffffffu, out);
-    }
-};
-
 // Walks the run's long chains (of the components of sh.team[0, teams), their
 // members among ranks [r0, r1)) with every warp of the CTA, no gap between long
 // tensors needing a look: the warps are dealt out to the chains, take their
 // chain's members in rank order in turn, each waits until its member's
 // predecessors are placed (the offsets it needs are what it polls), and places
 // it.  The lowest unplaced member's predecessors are placed and its warp has
-// nothing earlier left to do, so every wait ends; it is bounded all the same
-// (TeamWait, sh.fail).  A chain of equal sizes is deep but not a single path: 262 and 112
-// activations of a residual network, 172 K cycles by a warp each, 100 K this way.
+// nothing earlier left to do, so every wait ends; it is bounded all the same: a
+// warp that has polled kTeamPolls times counts the members that are placed, and
+// leaves (sh.fail) if they are no more than when it last did.  (One member may
+// keep the others waiting for some ms: one whose window is thousands of positions
+// wide goes through it once for every level it is stacked above.)  A chain of
+// equal sizes is deep but not a single path: 262 and 112 activations of a residual
+// network, 172 K cycles by a warp each, 100 K this way.
 __device__ __forceinline__ uint32_t walk_teams(const Ctx<false>& c, int32_t teams, int32_t r0, int32_t r1,
                                                const Longs& lg, Shared& sh) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -712,38 +693,53 @@ __device__ __forceinline__ uint32_t walk_teams(const Ctx<false>& c, int32_t team
     __syncthreads();
     uint32_t mx = 0;
     volatile unsigned long long* oe = reinterpret_cast<volatile unsigned long long*>(c.oe);
+    if (lane == 0) sh.seen[warp] = -1;
+    __syncwarp();
+    auto stuck = [&]() -> bool {  // (nothing of it is kept between calls: registers are short here)
+        int32_t now = 0;
+        for (int32_t x = first + lane; x < end; x += 32) now += oe[c.rec[c.list[x]].pos] != 0 ? 1 : 0;
+        now = __reduce_add_sync(full, now);
+        const bool out = __any_sync(full, now == *(volatile int32_t*)&sh.seen[warp] || *(volatile int32_t*)&sh.fail);
+        *(volatile int32_t*)(out ? &sh.fail : &sh.seen[warp]) = out ? 1 : now;
+        return out;
+    };
     for (int32_t i = first + warp % nwarps; i < end; i += nwarps) {
         const int32_t r = c.list[i];
         const Rec rc = c.rec[r];
         const Win w = c.win[r];
-        TeamWait wait;
-        uint32_t top;
+        bool out = false;
         if (w.wide) {  // no mask of its predecessors: every earlier member's turn first
-            for (int32_t x0 = first; x0 < i; x0 += 32) {
+            for (int32_t x0 = first; x0 < i && !out; x0 += 32) {
                 const bool pred = x0 + lane < i;
                 const int32_t q = pred ? c.rec[c.list[x0 + lane]].pos : 0;
-                for (int32_t polls = 0; __any_sync(full, pred && oe[q] == 0); ++polls)
-                    if (wait.over(sh, polls)) break;
+                for (int32_t polls = 0; !out && __any_sync(full, pred && oe[q] == 0); ++polls)
+                    if (polls > kTeamPolls) {
+                        out = stuck();
+                        polls = 0;
+                    }
             }
-            __syncwarp();
+            if (out) break;
             if (test_held(sh, rc.pos)) continue;
-            top = place_short(c, r, lg);
-        } else {
-            const bool pred = (c.mask[r] >> lane) & 1u;
-            const int32_t q = w.w0 + lane;
-            unsigned long long v = 0;
-            for (int32_t polls = 0;; ++polls) {
-                if (pred) v = oe[q];
-                if (!__any_sync(full, pred && v == 0)) break;
-                if (wait.over(sh, polls)) break;
-            }
-            if (test_held(sh, rc.pos)) continue;
-            const uint32_t o = fit_plain(make_uint2((uint32_t)v, (uint32_t)(v >> 32)), rc.s, lg.top, c.policy);
-            top = o + rc.s;
-            if (lane == 0) oe[rc.pos] = ((unsigned long long)top << 32) | o;
+            mx = umax2(mx, place_short(c, r, lg));
+            continue;
         }
-        if (lane == 0) *(volatile int32_t*)&sh.placed = r;
-        mx = umax2(mx, top);
+        const bool pred = (c.mask[r] >> lane) & 1u;
+        const int32_t q = w.w0 + lane;
+        unsigned long long v = 0;
+        for (int32_t polls = 0;; ++polls) {
+            if (pred) v = oe[q];
+            if (!__any_sync(full, pred && v == 0)) break;
+            if (polls > kTeamPolls) {
+                out = stuck();
+                if (out) break;
+                polls = 0;
+            }
+        }
+        if (out) break;
+        if (test_held(sh, rc.pos)) continue;
+        const uint32_t o = fit_plain(make_uint2((uint32_t)v, (uint32_t)(v >> 32)), rc.s, lg.top, c.policy);
+        if (lane == 0) oe[rc.pos] = ((unsigned long long)(o + rc.s) << 32) | o;
+        mx = umax2(mx, o + rc.s);
     }
     __syncthreads();
     return mx;
@@ -811,7 +807,7 @@ __device__ __forceinline__ uint32_t run_chains(const Ctx<kFar>& c, int32_t r0, i
         __syncthreads();
         if constexpr (!kFar) {
             const int32_t teams = min(sh.teams, kTeams);
-            if (teams > 0) mx = umax2(mx, walk_teams(c, teams, r0, r1, lg, sh));
+            if (teams > 0 && !sh.fail) mx = umax2(mx, walk_teams(c, teams, r0, r1, lg, sh));
         }
         const int32_t nh = sh.cnt, nh1 = sh.cnt1;
         // half of the warps begin with the long chains, half with the others
@@ -1358,7 +1354,6 @@ __device__ __forceinline__ bool plan(const mp_batch& bt, const TraceView& tv, in
         sh.bad = 0;
         sh.lw = 1;
         sh.fail = 0;
-        sh.placed = 0;
         sh.hold = out.hold;
         sh.hi = sh.lo = sh.bits = 0;
         sh.lb = sh.far = sh.last_free = 0;
