@@ -9,6 +9,7 @@
 #include <set>
 #include <tuple>
 #include <utility>
+#include <vector>
 
 #include "launch.h"
 #include "memplan.h"
@@ -316,3 +317,26 @@ __attribute__((visibility("default"))) mp_status mp_peak(const mp_batch* batch, 
 }
 
 }  // extern "C"
+
+#ifdef MP_TEST_HOOKS
+namespace mp {
+static std::vector<TestRouteReader>& test_route_readers() {
+    static std::vector<TestRouteReader> readers;
+    return readers;
+}
+bool test_add_routes(TestRouteReader reader) {
+    test_route_readers().push_back(reader);
+    return true;
+}
+}  // namespace mp
+
+// Test builds only: the traces each route (mp::TestRoute) has taken on the
+// current device since the last call; counts: mp::kRoutes words.
+extern "C" __attribute__((visibility("default"))) mp_status mp_test_routes(uint32_t* counts) {
+    for (int r = 0; r < mp::kRoutes; ++r) counts[r] = 0;
+    cudaError_t e = cudaDeviceSynchronize();
+    for (auto reader : mp::test_route_readers())
+        if (e == cudaSuccess) e = reader(counts);
+    return e == cudaSuccess ? MP_OK : MP_ECUDA;
+}
+#endif

@@ -34,7 +34,6 @@ namespace mp {
 
 namespace {
 
-constexpr size_t kTwoPerSm = 110 * 1024;  // shared memory of a CTA of which an SM holds two
 constexpr int32_t kBDeferred = -2;  // status of a trace left by k_breadth_comp to k_breadth_rest
 
 // Per-trace working set: the breadth of the operator at each step; per tensor
@@ -620,6 +619,7 @@ k_breadth_comp(mp_batch bt, int32_t policy, int64_t* __restrict__ offsets, int64
         if (tid == 0) status[b] = kBDeferred;
         return;
     }
+    test_route(kRouteBreadthComp);
     if (tid == 0) {  // thread-tier components in descending size: bin starts, then cursors; member counts
         int32_t at = 0, mat = 0;
         for (int32_t k = 0; k < kBThreadComp - 1; ++k) {
@@ -783,8 +783,10 @@ k_breadth_rest(mp_batch bt, int32_t policy, int64_t* __restrict__ offsets, int64
                     o.status = status + b;
                     o.hold = phases::test_team_hold(b);
                     done = phases::plan<true, false>(bt, tv, policy, o);
+                    if (done) test_route(kRouteBreadthPhases);
                 }
             }
+            if (!done && by_tensor) test_route(kRouteBreadthTensor);
             if (!done && by_tensor) breadth_trace<kSmem>(b, bt, policy, offsets, plan_peak, status, ws, ws_stride);
             if (!done && !by_tensor && threadIdx.x == 0) status[b] = kBDeferred;  // left to the next launch
             __syncthreads();

@@ -8,9 +8,29 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "launch.h"
 #include "memplan.h"
 
 namespace mp {
+
+// One trace took this route (called by the whole block; counted in test builds).
+#ifdef MP_TEST_HOOKS
+static __device__ unsigned g_test_routes[kRoutes];
+__device__ __forceinline__ void test_route(TestRoute r) {
+    if (threadIdx.x == 0) atomicAdd(&g_test_routes[r], 1u);
+}
+static cudaError_t test_read_routes(unsigned* counts) {
+    unsigned mine[kRoutes], none[kRoutes] = {};
+    cudaError_t e = cudaMemcpyFromSymbol(mine, g_test_routes, sizeof(mine));
+    if (e == cudaSuccess) e = cudaMemcpyToSymbol(g_test_routes, none, sizeof(none));
+    if (e == cudaSuccess)
+        for (int r = 0; r < kRoutes; ++r) counts[r] += mine[r];
+    return e;
+}
+static const bool g_test_routes_added = test_add_routes(&test_read_routes);
+#else
+__device__ __forceinline__ void test_route(TestRoute) {}
+#endif
 
 constexpr int kWarp = 32;
 constexpr uint64_t kSatCap = 0x8000000000000000ull;  // INT64_MAX + 1

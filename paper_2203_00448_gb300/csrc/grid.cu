@@ -1114,6 +1114,10 @@ k_grid_flow(mp_batch bt, int32_t policy, GridWs w, int32_t long_ctas) {
         return;
     }
 
+    if (blockIdx.x == 0)
+        for (int32_t b = 0; b < bt.n_traces; ++b)
+            if (w.ti[b].ok) test_route(kRouteGridFlow);
+
     // the long-lived cache: trace b's records at [s_cbase[b], s_cbase[b + 1])
     LongCache lc;
     {
@@ -1225,7 +1229,10 @@ __global__ void __launch_bounds__(kFarThreads, 1) k_grid_phases(mp_batch bt, int
     asm volatile("griddepcontrol.wait;" ::: "memory");  // for the flow kernel
     asm volatile("griddepcontrol.launch_dependents;");
     const TraceInfo* ti = w.ti + blockIdx.x;
-    if (ti->ok && in_phases(w.ctl) && w.ctl->fail == 0) far_place(w, (int32_t)blockIdx.x, policy, smem_raw, sh, fs);
+    if (ti->ok && in_phases(w.ctl) && w.ctl->fail == 0) {
+        test_route(kRouteGridPhases);
+        far_place(w, (int32_t)blockIdx.x, policy, smem_raw, sh, fs);
+    }
 }
 
 // ---------------------------------------------------------------- finish

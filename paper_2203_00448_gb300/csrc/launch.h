@@ -25,6 +25,7 @@ constexpr int kPlanThreadsWide = 512;    // the 64-bit launch: deferred traces, 
 // Largest dynamic shared memory a kernel of this library requests per CTA
 // (sm_103a allows 227 KB); above it a kernel keeps its data in the workspace.
 constexpr size_t kSmemCeiling = 200 * 1024;
+constexpr size_t kTwoPerSm = 110 * 1024;  // dynamic shared memory of a CTA of which an SM holds two
 constexpr size_t kProfileSmemLimit = kSmemCeiling;
 constexpr size_t kValidateSmemLimit = kSmemCeiling;
 constexpr size_t kPlanSmemLimit = kSmemCeiling;
@@ -39,6 +40,26 @@ cudaError_t max_resident_ctas(const void* func, int threads, size_t smem, int* c
 
 // SMs of the current device; cached per device.
 cudaError_t sm_count(int* sms);
+
+// Test builds (MP_TEST_HOOKS) count the traces each placement route has taken
+// (mp_test_routes); every translation unit has counters of its own and adds
+// itself to the list that abi.cu sums up.
+enum TestRoute {
+    kRouteFirst,          // first launch, no component past the warp tier
+    kRouteWalk,           // ... and some, walked
+    kRoutePhases,         // second launch, in phases
+    kRouteGeneral,        // ... by the general path
+    kRouteGridFlow,       // a few large traces: by the dataflow over the whole GPU
+    kRouteGridPhases,     // ... in phases
+    kRouteBreadthComp,    // by breadth: by components
+    kRouteBreadthPhases,  // ... in phases
+    kRouteBreadthTensor,  // ... tensor by tensor
+    kRoutes
+};
+#ifdef MP_TEST_HOOKS
+using TestRouteReader = cudaError_t (*)(unsigned* counts);  // adds its counts and clears them
+bool test_add_routes(TestRouteReader reader);
+#endif
 
 // Alignment of every workspace slice.
 constexpr size_t kAlign = 256;

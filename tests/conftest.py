@@ -23,3 +23,32 @@ def cuda_lib():
 
     build.build()
     return _lib.load()
+
+
+ROUTES = ("first", "walk", "phases", "general", "grid-flow", "grid-phases", "breadth-comp", "breadth-phases",
+          "breadth-tensor")  # mp::TestRoute
+
+
+@pytest.fixture
+def routes(cuda_lib):
+    """The package on a test build of the library that counts the traces each
+    placement route takes: yields a function that returns {route: traces} since
+    its last call, routes that took none left out."""
+    import ctypes
+
+    from paper_2203_00448_gb300 import _lib, build
+
+    path = build.build_test_hooks()
+    plain, _lib._lib = _lib._lib, None
+    try:
+        lib = _lib.load(path)
+        counts = (ctypes.c_uint32 * len(ROUTES))()
+
+        def read():
+            assert lib.mp_test_routes(counts) == 0
+            return {r: c for r, c in zip(ROUTES, counts) if c}
+
+        read()
+        yield read
+    finally:
+        _lib._lib = plain

@@ -1,0 +1,93 @@
+"""Which kernel places a trace, over the lines of the rules that choose it (the
+routes are counted in a test build of the library), and its results there
+against the oracle."""
+import numpy as np
+import pytest
+
+import tracegen as tg
+
+from tests.test_gpu_phases import _check, _trace
+
+pytestmark = pytest.mark.gpu
+
+
+def _linked(rng, n, sizes=64, life=3):
+    """One component of n tensors without long-lived ones: each overlaps the next."""
+    a = np.arange(n)
+    return n + life + 1, a, a + rng.integers(2, life + 1, size=n), rng.integers(1, sizes + 1, size=n) * 256
+
+
+def _small(rng):
+    return _trace(rng, 40, 40, 0.0, 64, 1 << 14)
+
+
+def _plans(ts, routes):
+    """Routes of one call per policy of the planner by size, and by breadth."""
+    import paper_2203_00448_gb300 as mp
+
+    db = mp.DeviceBatch.from_host(ts, "cuda")
+    got = []
+    for fn in (mp.plan_and_validate, mp.plan_greedy_by_size, mp.plan_greedy_by_breadth):
+        for policy in ("first", "best"):
+            fn(db, policy)
+            got.append(routes())
+    assert all(g == got[0] for g in got[:4]), got
+    return got[0], got[4], got[5]
+
+
+# (traces, members of the component, route): 34 traces and 310 are on either side of what the phases hold at once
+@pytest.mark.parametrize("traces,n,route", ((34, 65, "walk"), (34, 128, "walk"), (34, 129, "phases"), (310, 65, "walk"),
+                                            (34, 200, "phases"), (310, 129, "walk"), (310, 1023, "walk"),
+                                            (310, 1024, "walk"), (310, 1025, "phases")))
+def test_chains(routes, traces, n, route):
+    rng = np.random.default_rng(n + traces)
+    ts = tg.from_arrays([_linked(rng, n if k % 16 == 0 else 30, (3, 1 << 12)[k // 16 % 2]) for k in range(traces)])
+    big = (traces + 15) // 16
+    size, _, _ = _plans(ts, routes)
+    assert size == {"first": traces - big, route: big}
+    _check(ts)
+
+
+# a step's tensors: windows of 2.8 times as many positions on average, on either side of the rule's line
+@pytest.mark.parametrize("traces,per_step,route", ((34, 16, "phases"), (310, 46, "walk"), (310, 47, "phases"),
+                                                   (1000, 46, "walk")))
+def test_wide_windows(routes, traces, per_step, route):
+    rng = np.random.default_rng(per_step + traces)
+    ts = []
+    for k in range(traces):
+        if k % 50:
+            ts.append(_small(rng))
+            continue
+        a = np.repeat(np.arange(10), per_step)  # each lives two steps
+        ts.append((12, a, a + 2, rng.integers(1, 1 << 10, len(a)) * 64))
+    big = (traces + 49) // 50
+    ts = tg.from_arrays(ts)
+    size, _, _ = _plans(ts, routes)
+    assert size == {"first": traces - big, route: big}
+    _check(ts)
+
+
+def test_long_lived_members_are_not_walked(routes):
+    rng = np.random.default_rng(1)
+    ts = [_small(rng) for _ in range(320)]
+    T, a, f, s = _linked(rng, 200)
+    f[50] = a[50] + 32  # the longest a short-lived tensor lives
+    ts[3] = (T, a, f, s)
+    T, a, f, s = _linked(rng, 200)
+    f[50] = a[50] + 33
+    ts[7] = (T, a, f, s)
+    ts = tg.from_arrays(ts)
+    size, _, _ = _plans(ts, routes)
+    assert size == {"first": 318, "walk": 1, "phases": 1}
+    _check(ts)
+
+
+@pytest.mark.parametrize("T,route", ((400, "walk"), (401, "phases")))
+def test_sparse_batches_do_not_walk(routes, T, route):
+    """Fewer than three tensors in four steps (by the longest trace): the kernel without the walk."""
+    rng = np.random.default_rng(2)
+    _, a, f, s = _linked(rng, 300)
+    ts = tg.from_arrays([_small(rng) for _ in range(310)] + [(T, a, f, s)])
+    size, _, _ = _plans(ts, routes)
+    assert size == {"first": 310, route: 1}
+    _check(ts)
