@@ -748,14 +748,14 @@ k_breadth_comp(mp_batch bt, int32_t policy, int64_t* __restrict__ offsets, int64
 }
 
 // The traces k_breadth_comp deferred (or, with deferred_only false, all of
-// them), in phases where they fit that path (in_phases: the batch may), else
-// tensor by tensor (by_tensor; otherwise they are left deferred).  It waits for
+// them), in phases where they fit that path (phase_smem: the shared memory for
+// it; 0: none does), else tensor by tensor (by_tensor; otherwise they are left deferred).  It waits for
 // the kernel before it in the kernel.
 template <bool kSmem>
 __global__ void __launch_bounds__(kBreadthPhaseThreads, 1)
 k_breadth_rest(mp_batch bt, int32_t policy, int64_t* __restrict__ offsets, int64_t* __restrict__ plan_peak,
                int32_t* __restrict__ status, unsigned char* __restrict__ ws, size_t ws_stride, bool deferred_only,
-               bool in_phases, bool by_tensor) {
+               uint32_t phase_smem, bool by_tensor) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;");
     // this CTA's traces are blockIdx.x + k * gridDim.x; their statuses are
@@ -774,9 +774,9 @@ k_breadth_rest(mp_batch bt, int32_t policy, int64_t* __restrict__ offsets, int64
         for (; m; m &= m - 1) {
             const int b = (int)(blockIdx.x + (k0 + __ffs(m) - 1) * gridDim.x);
             bool done = false;
-            if (in_phases) {
+            if (phase_smem > 0) {
                 const TraceView tv = load_trace(bt, b, false);
-                if (tv.st == MP_OK) {
+                if (tv.st == MP_OK && phases::fits<true>(tv.n, tv.T, phase_smem)) {
                     phases::Out o = {};
                     o.offsets = offsets + tv.lo;
                     o.plan_peak = plan_peak + b;
@@ -801,16 +801,17 @@ bool breadth_comp_fits(const mp_batch& bt) {
 // One launch of k_breadth_rest: in phases, tensor by tensor, or both.
 template <bool kSmem>
 cudaError_t launch_rest_once(const mp_batch& bt, int32_t policy, int64_t* offsets, int64_t* plan_peak, int32_t* status,
-                             void* workspace, bool deferred_only, bool in_phases, bool by_tensor,
+                             void* workspace, bool deferred_only, size_t phase_smem, bool by_tensor,
                              cudaStream_t stream) {
     const size_t data = BreadthLayout(bt.max_tensors, bt.max_steps).total;
     size_t smem = kSmem && by_tensor ? data : 0;
-    if (in_phases) smem = std::max(smem, phases::smem_bytes<true>(bt));
+    smem = std::max(smem, phase_smem);
     const void* fn = (const void*)k_breadth_rest<kSmem>;
     int sms = 0, resident = 0;
     cudaError_t e = sm_count(&sms);
-    // more traces than SMs: half the threads, so that an SM holds two
-    const int threads = bt.n_traces > sms ? kBreadthPhaseThreads / 2 : kBreadthPhaseThreads;
+    // more traces than SMs: half the threads, where an SM holds two of them
+    const int threads =
+        bt.n_traces > sms && smem <= kTwoPerSm ? kBreadthPhaseThreads / 2 : kBreadthPhaseThreads;
     if (e == cudaSuccess) e = set_smem_limit(fn, smem);
     if (e == cudaSuccess) e = max_resident_ctas(fn, threads, smem, &resident);
     if (e != cudaSuccess) return e;
@@ -825,7 +826,8 @@ cudaError_t launch_rest_once(const mp_batch& bt, int32_t policy, int64_t* offset
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, k_breadth_rest<kSmem>, bt, policy, offsets, plan_peak, status,
-                              static_cast<unsigned char*>(workspace), data, deferred_only, in_phases, by_tensor);
+                              static_cast<unsigned char*>(workspace), data, deferred_only, (uint32_t)phase_smem,
+                              by_tensor);
 }
 
 // Both ways in one launch where that leaves room for two CTAs an SM, else one
@@ -833,15 +835,15 @@ cudaError_t launch_rest_once(const mp_batch& bt, int32_t policy, int64_t* offset
 // the 160 KB that placing one of them tensor by tensor would need.
 template <bool kSmem>
 cudaError_t launch_rest(const mp_batch& bt, int32_t policy, int64_t* offsets, int64_t* plan_peak, int32_t* status,
-                        void* workspace, bool deferred_only, bool in_phases, cudaStream_t stream) {
+                        void* workspace, bool deferred_only, size_t phase_smem, cudaStream_t stream) {
     const size_t data = BreadthLayout(bt.max_tensors, bt.max_steps).total;
-    if (kSmem && in_phases && data > std::max(phases::smem_bytes<true>(bt), kTwoPerSm)) {
+    if (kSmem && phase_smem > 0 && data > std::max(phase_smem, kTwoPerSm)) {
         const cudaError_t e = launch_rest_once<kSmem>(bt, policy, offsets, plan_peak, status, workspace, deferred_only,
-                                                      true, false, stream);
+                                                      phase_smem, false, stream);
         if (e != cudaSuccess) return e;
-        return launch_rest_once<kSmem>(bt, policy, offsets, plan_peak, status, workspace, true, false, true, stream);
+        return launch_rest_once<kSmem>(bt, policy, offsets, plan_peak, status, workspace, true, 0, true, stream);
     }
-    return launch_rest_once<kSmem>(bt, policy, offsets, plan_peak, status, workspace, deferred_only, in_phases, true,
+    return launch_rest_once<kSmem>(bt, policy, offsets, plan_peak, status, workspace, deferred_only, phase_smem, true,
                                    stream);
 }
 
@@ -855,18 +857,23 @@ size_t breadth_workspace_bytes(const mp_batch& bt) {
 cudaError_t launch_breadth(const mp_batch& bt, int32_t policy, int64_t* offsets, int64_t* plan_peak, int32_t* status,
                            void* workspace, cudaStream_t stream) {
     if (bt.n_traces == 0) return cudaSuccess;
-    const bool comp = breadth_comp_fits(bt), in_phases = phases::batch_fits<true>(bt);
+    const bool comp = breadth_comp_fits(bt);
+    int sms = 0;
+    cudaError_t e = sm_count(&sms);
+    if (e != cudaSuccess) return e;
+    const size_t phase_smem = phases::smem_bytes<true>(bt, sms);
     if (comp) {
         const size_t cbytes = BCompLayout(bt.max_tensors, bt.max_steps).total;
-        cudaError_t e = set_smem_limit((const void*)k_breadth_comp, cbytes);
+        e = set_smem_limit((const void*)k_breadth_comp, cbytes);
         if (e != cudaSuccess) return e;
         k_breadth_comp<<<(unsigned)bt.n_traces, kBreadthThreads, cbytes, stream>>>(bt, policy, offsets, plan_peak,
-                                                                                  status, in_phases);
+                                                                                  status, phase_smem > 0);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
-    return breadth_fits_smem(bt) ? launch_rest<true>(bt, policy, offsets, plan_peak, status, workspace, comp, in_phases, stream)
-                                 : launch_rest<false>(bt, policy, offsets, plan_peak, status, workspace, comp, in_phases, stream);
+    return breadth_fits_smem(bt)
+               ? launch_rest<true>(bt, policy, offsets, plan_peak, status, workspace, comp, phase_smem, stream)
+               : launch_rest<false>(bt, policy, offsets, plan_peak, status, workspace, comp, phase_smem, stream);
 }
 
 }  // namespace mp

@@ -41,12 +41,14 @@ namespace phases {
 
 constexpr int32_t kLong = 32;          // lives above this many steps are long
 constexpr int32_t kMaxLong = 768;      // long tensors a trace may have here
-constexpr int32_t kMaxTensors = 4096;  // tensors a trace may have here
+constexpr int32_t kMaxTensors = 4080;  // tensors a trace may have here: no more fit the shared memory (Layout)
 constexpr uint32_t kLongestChain = 1024;  // positions a chain may span beside long tensors: one warp walks it, the
                                        // general paths' queues place its members side by side
+constexpr int32_t kMixedTensors = 1024;  // most tensors a trace may have on average in a batch of mixed lengths (smem_bytes)
 constexpr int32_t kBatch = 512;        // tensors inserted into the sorted list at a time
 constexpr int32_t kHeads = 1024;       // chains of a run listed at a time
-constexpr int32_t kChunk = 16;         // sorted-list entries per thread: kMaxTensors / the fewest threads
+constexpr int32_t kChunk = 8;          // sorted-list entries per thread, at most: the callers have 512 threads, or 256
+                                       // where an SM holds two CTAs, whose traces have 2,048 tensors at most
 constexpr int32_t kNear = 32;          // neighbours listed per short tensor of a large trace (grid_phases.cuh)
 constexpr int32_t kThreadChain = 8;    // chains up to this long within a run can be walked by one thread
 constexpr int32_t kTeamChain = 64;     // chains from this length on are walked by the whole CTA together ...
@@ -87,14 +89,15 @@ struct __align__(8) Win {
 // differences, the operators' breadths), then the records; bucket ends, then
 // the long tensors and the scratch of insertions; sizes, then the windows.
 struct Layout {
-    size_t oe, rec, win, mask, af, id, sl, tmp, bend, lg_oe, lg_af, lr, pk, heads, total;
+    size_t oe = 0, rec = 0, win = 0, mask = 0, af = 0, id = 0, sl = 0, tmp = 0, bend = 0;
+    size_t lg_oe = 0, lg_af = 0, lr = 0, pk = 0, heads = 0, total = 0;
     __host__ __device__ static constexpr size_t a16(size_t x) { return (x + 15) & ~size_t(15); }
     __host__ __device__ static constexpr int32_t keys_of(int32_t n) {  // sort length
         int32_t k = 512;  // a key per thread at least
         while (k < n) k <<= 1;
         return k;
     }
-    __host__ __device__ Layout(int32_t n, int32_t T, size_t step_bytes) {
+    __host__ __device__ constexpr Layout(int32_t n, int32_t T, size_t step_bytes) {
         oe = 0;
         rec = oe + (size_t)keys_of(n) * 8;
         const size_t recs = a16((size_t)n * sizeof(Rec)), steps = a16((size_t)T * step_bytes);
@@ -122,22 +125,36 @@ __host__ __device__ constexpr size_t step_bytes() {
     return kBreadth ? 8 : 4;
 }
 
-// Shared memory for any trace of the batch, and whether the batch's host
-// scalars keep every trace within the limits.
+static_assert(Layout(kMaxTensors, 1, 4).total <= kSmemCeiling && Layout(kMaxTensors + 1, 1, 4).total > kSmemCeiling,
+              "the most tensors a trace may have");
+static_assert(kMaxTensors <= 512 * kChunk && Layout(256 * kChunk + 1, 1, 4).total > kTwoPerSm,
+              "the sorted list's entries are held in registers while some are inserted");
+
+// Whether a trace of n tensors over T steps can be placed here with that much
+// dynamic shared memory.
 template <bool kBreadth>
-size_t smem_bytes(const mp_batch& bt) {
-    return Layout(bt.max_tensors, bt.max_steps, step_bytes<kBreadth>()).total;
+__host__ __device__ bool fits(int32_t n, int32_t T, size_t smem) {
+    return n <= kMaxTensors && T <= 65535 && Layout(n, T, step_bytes<kBreadth>()).total <= smem;
 }
+
+// Dynamic shared memory that a launch for the batch's traces should have: enough
+// for the longest; where that is too much, as in a batch of ordinary traces with
+// a very long one among them, what leaves an SM as many CTAs as the batch can
+// use, and the traces it holds are placed here (600 chains of 374 tensors and a
+// trace of 2,000 over 20,000 steps: MIXEDUS); 0 if few would be.
 template <bool kBreadth>
-bool batch_fits(const mp_batch& bt) {
-    return bt.max_tensors <= kMaxTensors && bt.max_steps <= 65535 && smem_bytes<kBreadth>(bt) <= kSmemCeiling;
+size_t smem_bytes(const mp_batch& bt, int sms) {
+    if (fits<kBreadth>(bt.max_tensors, bt.max_steps, kSmemCeiling))
+        return Layout(bt.max_tensors, bt.max_steps, step_bytes<kBreadth>()).total;
+    if (bt.n_tensors / bt.n_traces > kMixedTensors) return 0;
+    return bt.n_traces > sms ? kTwoPerSm : kSmemCeiling;
 }
 
 struct Shared {
     uint32_t red[33];
     unsigned long long hi, lo, bits, best;
     uint32_t best32, lb, far;
-    int32_t bad, lw, cnt, next, cnt1, next1, teams, fail;
+    int32_t bad, lw, nl, cnt, next, cnt1, next1, teams, fail;
     int32_t seen[16];  // by warp: members of its team placed when it last asked
     int32_t hold;    // test builds: alloc-order position of a team's member that is never placed (-1: none)
     uint16_t team[kTeams];
@@ -1313,17 +1330,17 @@ static __device__ __noinline__ void sort_keys(int32_t n) {
     if (n <= nt) go(std::integral_constant<int, 1>());
     else if (n <= 2 * nt) go(std::integral_constant<int, 2>());
     else if (n <= 4 * nt) go(std::integral_constant<int, 4>());
-    else if (n <= 8 * nt) go(std::integral_constant<int, 8>());
-    else go(std::integral_constant<int, 16>());
+    else go(std::integral_constant<int, 8>());  // (kChunk)
 }
 
 // The whole trace by the whole CTA (256 or 512 threads): checks, profile (when
 // out.profile is set), priority order (greedy_by_size, or greedy by breadth
 // with kBreadth), placement, validation (kCheck) and outputs.  Returns false,
-// with nothing but the profile written, when the trace is not one for this
-// path: an invalid tensor, sizes summing to 2^32 units or more, too many long
-// tensors, or a long chain beside some.  Either way no thread touches the
-// dynamic shared memory any more when another one returns.
+// with nothing written, when the trace is not one for this path: an invalid
+// tensor, sizes summing to 2^32 units or more, too many long tensors, or a long
+// chain beside some.  That is known before the sorts, so that a trace for the
+// general path loses little here (REFUSEDUS), and no thread touches the dynamic
+// shared memory any more when another one returns.
 template <bool kBreadth, bool kCheck>
 __device__ __forceinline__ bool plan(const mp_batch& bt, const TraceView& tv, int32_t policy, const Out& out) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1351,7 +1368,7 @@ __device__ __forceinline__ bool plan(const mp_batch& bt, const TraceView& tv, in
     // ---- checks, size sum and unit, alloc-step histogram
     for (int32_t i = t; i < T; i += nt) BEND[i] = 0;
     if (t == 0) {
-        sh.bad = 0;
+        sh.bad = sh.nl = 0;
         sh.lw = 1;
         sh.fail = 0;
         sh.hold = out.hold;
@@ -1363,6 +1380,7 @@ __device__ __forceinline__ bool plan(const mp_batch& bt, const TraceView& tv, in
     {
         bool bad = false;
         uint64_t sum = 0, bits = 0;
+        int32_t longs = 0;
         for (int32_t k = t; k < n; k += nt) {
             const int32_t a = __ldg(Ag + k), f = __ldg(Fg + k);
             const int64_t s = __ldg(Sg + k);
@@ -1370,6 +1388,7 @@ __device__ __forceinline__ bool plan(const mp_batch& bt, const TraceView& tv, in
                 bad = true;
                 continue;
             }
+            longs += f - a > kLong ? 1 : 0;
             sum = sat_add(sum, (uint64_t)s);
             bits |= (uint64_t)s;
             KEY[k] = (uint64_t)s;
@@ -1379,11 +1398,16 @@ __device__ __forceinline__ bool plan(const mp_batch& bt, const TraceView& tv, in
         block_add_size_sum(sum, &sh.hi, &sh.lo);
         const unsigned b0 = __reduce_or_sync(0xffffffffu, (unsigned)bits);
         const unsigned b1 = __reduce_or_sync(0xffffffffu, (unsigned)(bits >> 32));
-        if (lane == 0) atomicOr(&sh.bits, ((unsigned long long)b1 << 32) | b0);
+        longs = __reduce_add_sync(0xffffffffu, longs);
+        if (lane == 0) {
+            atomicOr(&sh.bits, ((unsigned long long)b1 << 32) | b0);
+            if (longs) atomicAdd(&sh.nl, longs);
+        }
         if (bad) sh.bad = 1;
     }
     __syncthreads();
-    if (sh.bad || n == 0 || size_sum_overflows(sh.hi, sh.lo)) return false;
+    const int32_t nl = sh.nl;
+    if (sh.bad || n == 0 || size_sum_overflows(sh.hi, sh.lo) || nl > kMaxLong) return false;
     const int shift = __ffsll((long long)sh.bits) - 1;
     if ((((sh.hi << 32) + sh.lo) >> shift) > 0xffffffffull) return false;
 
@@ -1433,6 +1457,44 @@ __device__ __forceinline__ bool plan(const mp_batch& bt, const TraceView& tv, in
         }
     }
     __syncthreads();
+
+    // ---- components of short lifetimes linked by overlap: one starts at a short
+    // tensor allocated when every earlier short one is freed.  SL[q]: 1 + the first
+    // position of q's component (0: q is long).
+    {
+        const int32_t chunk = (n + nt - 1) / nt, q0 = min(n, t * chunk), q1 = min(n, q0 + chunk);
+        auto is_short = [](uint32_t af) { return (int32_t)(af >> 16) - (int32_t)(af & 0xffffu) <= kLong; };
+        uint32_t live = 0;
+        for (int32_t q = q0; q < q1; ++q)
+            if (is_short(AF[q])) live = umax2(live, AF[q] >> 16);
+        uint32_t tot;
+        const uint32_t before = block_excl_max(live, sh.red, &tot);
+        uint32_t run = before, start = 0;  // start: 1 + position of the last component start
+        for (int32_t q = q0; q < q1; ++q) {
+            const uint32_t af = AF[q];
+            if (!is_short(af)) continue;
+            if (run <= (af & 0xffffu)) start = (uint32_t)q + 1;
+            run = umax2(run, af >> 16);
+        }
+        start = block_excl_max(start, sh.red, &tot);
+        run = before;
+        // the longest stretch of positions of one component bounds the work of
+        // looking through it member by member
+        uint32_t far = 0;
+        for (int32_t q = q0; q < q1; ++q) {
+            const uint32_t af = AF[q];
+            SL[q] = 0;
+            if (!is_short(af)) continue;
+            if (run <= (af & 0xffffu)) start = (uint32_t)q + 1;
+            run = umax2(run, af >> 16);
+            SL[q] = (uint16_t)start;
+            far = umax2(far, (uint32_t)q + 1 - start);
+        }
+        far = __reduce_max_sync(0xffffffffu, far);
+        if (lane == 0 && far) atomicMax(&sh.far, far);
+    }
+    __syncthreads();
+    if (nl > 0 && sh.far > kLongestChain) return false;
 
     // ---- live profile: prefix sums of the differences
     if (want_profile) {
@@ -1523,44 +1585,8 @@ __device__ __forceinline__ bool plan(const mp_batch& bt, const TraceView& tv, in
         MASK[r] = mask;
     }
 
-    // ---- chains: components of short lifetimes linked by overlap, each in
-    // rank order.  A component starts at a short tensor allocated when every
-    // earlier short one is freed.
-    {
-        const int32_t chunk = (n + nt - 1) / nt, q0 = min(n, t * chunk), q1 = min(n, q0 + chunk);
-        auto is_short = [](uint32_t af) { return (int32_t)(af >> 16) - (int32_t)(af & 0xffffu) <= kLong; };
-        uint32_t live = 0;
-        for (int32_t q = q0; q < q1; ++q)
-            if (is_short(AF[q])) live = umax2(live, AF[q] >> 16);
-        uint32_t tot;
-        const uint32_t before = block_excl_max(live, sh.red, &tot);
-        uint32_t run = before, start = 0;  // start: 1 + position of the last component start
-        for (int32_t q = q0; q < q1; ++q) {
-            const uint32_t af = AF[q];
-            if (!is_short(af)) continue;
-            if (run <= (af & 0xffffu)) start = (uint32_t)q + 1;
-            run = umax2(run, af >> 16);
-        }
-        start = block_excl_max(start, sh.red, &tot);
-        run = before;
-        for (int32_t q = q0; q < q1; ++q) {
-            const uint32_t af = AF[q];
-            if (!is_short(af)) {
-                KEY[q] = kLongKey;
-                continue;
-            }
-            if (run <= (af & 0xffffu)) start = (uint32_t)q + 1;
-            run = umax2(run, af >> 16);
-            KEY[q] = ((uint64_t)start << 16) | TMP[q];
-        }
-        // the longest stretch of positions of one component bounds the work of
-        // looking through it member by member
-        uint32_t far = 0;
-        for (int32_t q = q0; q < q1; ++q)
-            if (KEY[q] != kLongKey) far = umax2(far, (uint32_t)q + 1 - (uint32_t)(KEY[q] >> 16));
-        far = __reduce_max_sync(0xffffffffu, far);
-        if (lane == 0 && far) atomicMax(&sh.far, far);
-    }
+    // ---- chains: the components, each in rank order
+    for (int32_t q = t; q < n; q += nt) KEY[q] = SL[q] ? ((uint64_t)SL[q] << 16) | TMP[q] : kLongKey;
     __syncthreads();
     if (sh.far * (uint32_t)((n + nt - 1) / nt) < kScanChain) {  // each member looks for its neighbours in rank among the others
         for (int32_t q = t; q < n; q += nt) {
@@ -1593,21 +1619,16 @@ __device__ __forceinline__ bool plan(const mp_batch& bt, const TraceView& tv, in
         }
     }
     __syncthreads();
-    int32_t nl = 0;
     // ---- ranks of the long tensors (the bucket ends are dead), offsets cleared
     uint16_t* LR = reinterpret_cast<uint16_t*>(smem + L.lr);
-    for (int32_t r0 = 0; r0 < n; r0 += nt) {
+    for (int32_t r0 = 0, at0 = 0; r0 < n; r0 += nt) {
         const int32_t r = r0 + t;
         const uint32_t flag = r < n && REC[r].prev == kIsLong ? 1u : 0u;
         uint32_t tot;
-        const uint32_t at = (uint32_t)nl + block_excl_sum(flag, sh.red, &tot);
-        if (flag && at < (uint32_t)kMaxLong) LR[at] = (uint16_t)r;
-        nl += (int32_t)tot;
+        const uint32_t at = (uint32_t)at0 + block_excl_sum(flag, sh.red, &tot);
+        if (flag) LR[at] = (uint16_t)r;
+        at0 += (int32_t)tot;
     }
-    // every thread's ranks are written before the caller's general path takes
-    // the shared memory over
-    __syncthreads();
-    if (nl > kMaxLong || (nl > 0 && sh.far > kLongestChain)) return false;
     for (int32_t p = t; p < n; p += nt) OE[p] = make_uint2(0, 0);
     __syncthreads();
 

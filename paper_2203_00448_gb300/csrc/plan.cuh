@@ -2087,10 +2087,11 @@ __device__ __forceinline__ void plan_trace(const int b, const mp_batch& bt, cons
 // A deferred trace placed in phases (phases.cuh); false if it is not one for
 // that path.
 template <bool kFused>
-__device__ __forceinline__ bool plan_in_phases(const int b, const mp_batch& bt, const PlanOut& out) {
+__device__ __forceinline__ bool plan_in_phases(const int b, const mp_batch& bt, const PlanOut& out,
+                                               uint32_t phase_smem) {
     if (test_hold_position(b) >= 0) return false;  // a test holds back a member of the queue
     const TraceView tv = load_trace(bt, b, kFused && out.profile != nullptr);
-    if (tv.st != MP_OK) return false;
+    if (tv.st != MP_OK || !phases::fits<false>(tv.n, tv.T, phase_smem)) return false;
     phases::Out o = {};
     o.offsets = out.offsets + tv.lo;
     o.plan_peak = out.plan_peak + b;
@@ -2114,7 +2115,7 @@ __device__ __forceinline__ bool plan_in_phases(const int b, const mp_batch& bt, 
 template <typename I, typename W, bool kSmem, bool kFused, int kThreads, Tier kTier>
 __global__ void __launch_bounds__(kThreads, sizeof(W) == 8 || !kSmem ? 1 : kThreads == kPlanThreadsFew ? 2 : kPlanCtasSmem)
 k_plan(mp_batch bt, PlanOut out, unsigned char* __restrict__ ws, size_t data_stride, size_t buf_offset,
-       size_t buf_stride, bool in_phases, WalkRule rule) {
+       size_t buf_stride, uint32_t phase_smem, WalkRule rule) {
     if constexpr (sizeof(W) == 4) {
         // once every CTA of this grid runs, those of the 64-bit launch may take
         // what room is left; they wait for this grid to finish (and its writes
@@ -2139,7 +2140,7 @@ k_plan(mp_batch bt, PlanOut out, unsigned char* __restrict__ ws, size_t data_str
                 const int b = (int)(blockIdx.x + (k0 + __ffs(m) - 1) * gridDim.x);
                 m &= m - 1;
                 bool done = false;
-                if constexpr (sizeof(I) == 2) done = in_phases && plan_in_phases<kFused>(b, bt, out);
+                if constexpr (sizeof(I) == 2) done = phase_smem > 0 && plan_in_phases<kFused>(b, bt, out, phase_smem);
                 if (!done)
                     plan_trace<I, W, kSmem, kFused, kTier>(b, bt, out, ws, data_stride, buf_offset, buf_stride, rule);
                 __syncthreads();
@@ -2213,8 +2214,9 @@ PlanWorkspace plan_workspace(const mp_batch& bt) {
 template <bool kFused>
 WalkRule walk_rule(const mp_batch& bt, int sms) {
     const PlanGeometry wide = plan_geometry<int64_t>(bt, kFused);
-    if (!wide.narrow || !phases::batch_fits<false>(bt)) return {kWalkComp, kWalkComp};
-    const size_t smem = std::max(wide.smem ? wide.data : flow_smem_bytes<int64_t>(), phases::smem_bytes<false>(bt));
+    const size_t phase_smem = wide.narrow ? phases::smem_bytes<false>(bt, sms) : 0;
+    if (phase_smem == 0) return {kWalkComp, kWalkComp};
+    const size_t smem = std::max(wide.smem ? wide.data : flow_smem_bytes<int64_t>(), phase_smem);
     if (bt.n_traces <= (smem <= kTwoPerSm ? 2 * sms : sms))
         return {bt.max_tensors <= kWalkFew ? kWalkFew : kWarpComp, kWalkComp};
     return {kWalkComp, kWalkWindow};
@@ -2230,11 +2232,11 @@ cudaError_t launch_variant(const mp_batch& bt, const PlanGeometry& g, const Plan
         const cudaError_t e = sm_count(&sms);
         if (e != cudaSuccess) return e;
     }
-    const bool in_phases = sizeof(W) == 8 && sizeof(I) == 2 && phases::batch_fits<false>(bt);
-    if (in_phases) {
-        smem = std::max(smem, phases::smem_bytes<false>(bt));
-        if (bt.n_traces > sms) threads /= 2;  // more traces than SMs: half the threads, so that an SM holds two
-    }
+    // for the traces that are placed in phases (0: none)
+    const size_t phase_smem = sizeof(W) == 8 && sizeof(I) == 2 ? phases::smem_bytes<false>(bt, sms) : 0;
+    smem = std::max(smem, phase_smem);
+    // more traces than SMs: half the threads, where an SM holds two of them
+    if (phase_smem > 0 && bt.n_traces > sms && smem <= kTwoPerSm) threads /= 2;
     const WalkRule rule = kTier == kTierWalk ? walk_rule<kFused>(bt, sms) : WalkRule{0, 0};
     const void* fn = (const void*)k_plan<I, W, kSmem, kFused, kThreads, kTier>;
     {
@@ -2250,7 +2252,7 @@ cudaError_t launch_variant(const mp_batch& bt, const PlanGeometry& g, const Plan
     }
     if (sizeof(W) == 4) {
         k_plan<I, W, kSmem, kFused, kThreads, kTier><<<(unsigned)grid, threads, smem, stream>>>(
-            bt, out, ws, g.data_stride, pw.buf_offset, pw.buf_stride, false, rule);
+            bt, out, ws, g.data_stride, pw.buf_offset, pw.buf_stride, 0, rule);
         return cudaGetLastError();
     }
     // the 64-bit launch depends on the 32-bit one programmatically: its CTAs
@@ -2266,7 +2268,7 @@ cudaError_t launch_variant(const mp_batch& bt, const PlanGeometry& g, const Plan
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, k_plan<I, W, kSmem, kFused, kThreads, kTier>, bt, out, ws, g.data_stride, pw.buf_offset,
-                              pw.buf_stride, in_phases, rule);
+                              pw.buf_stride, (uint32_t)phase_smem, rule);
 }
 
 template <typename W, bool kFused>

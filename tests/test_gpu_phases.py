@@ -67,10 +67,10 @@ def test_phases_limits(cuda_lib, case):
     rng = np.random.default_rng(len(case))
     traces = [_trace(rng, 50, 100, 0.1, 64, 1 << 14) for _ in range(33)]
     for full in (False, True):
-        if case == "largest":
-            traces.append(_trace(rng, 4096, 6000, 0.05, 64, 1 << 16, full_span=full))
+        if case == "largest":  # the most tensors that fit the shared memory, and the most steps with them
+            traces.append(_trace(rng, 4080, 4248, 0.05, 64, 1 << 16, full_span=full))
         elif case == "too-many-tensors":  # past the path's limit: the general path
-            traces.append(_trace(rng, 4100, 6000, 0.03, 64, 1 << 16, full_span=full))
+            traces.append(_trace(rng, 4081, 3000, 0.03, 64, 1 << 16, full_span=full))
         elif case == "too-many-long":  # 768 fit, more are left to the general path
             for nl in (768, 769):
                 T, a, f, s = _trace(rng, 1000, 1200, 0.0, 64, 1 << 10)

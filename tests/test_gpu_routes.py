@@ -91,3 +91,62 @@ def test_sparse_batches_do_not_walk(routes, T, route):
     size, _, _ = _plans(ts, routes)
     assert size == {"first": 310, route: 1}
     _check(ts)
+
+
+# the most tensors the phases take, with the most steps; and the most of a launch that has 256 threads a trace
+@pytest.mark.parametrize("traces,n,T,route", ((34, 4080, 4248, "phases"), (34, 4080, 4249, "general"), (34, 4081, 300, "general"),
+                                              (160, 2048, 2400, "phases"), (160, 2049, 2400, "phases"),
+                                              (160, 4080, 4248, "phases")))
+def test_phases_limits(routes, traces, n, T, route):
+    rng = np.random.default_rng(n + T)
+    ts = [_small(rng) for _ in range(traces)]
+    for k in (1, traces - 1):
+        ts[k] = _trace(rng, n, T, 0.05, 64, 1 << 14, full_span=k > 1)
+    ts = tg.from_arrays(ts)
+    size, first, best = _plans(ts, routes)
+    assert size == {"first": traces - 2, route: 2}
+    other = {"phases": "breadth-phases", "general": "breadth-tensor"}[route]
+    assert first == best and first[other] == 2 if other == "breadth-tensor" else first[other] >= 2
+    _check(ts)
+
+
+@pytest.mark.parametrize("traces", (40, 160))
+def test_a_long_trace_among_ordinary_ones(routes, traces):
+    """One trace past the phases' limits leaves them to the others."""
+    rng = np.random.default_rng(traces)
+    ts = [_small(rng) for _ in range(traces)]
+    for k in (0, 5, 9):
+        ts[k] = _trace(rng, 500, 600, 0.05, 64, 1 << 14, full_span=k > 0)
+    ts[3] = _trace(rng, 2000, 20000, 0.0, 64, 1 << 14)  # steps
+    ts[4] = _trace(rng, 5000, 4000, 0.02, 64, 1 << 14, full_span=True)  # tensors
+    ts = tg.from_arrays(ts)
+    size, first, best = _plans(ts, routes)
+    assert size == {"first": traces - 4, "phases": 3, "general": 1}
+    assert first == best and first["breadth-phases"] >= 3
+    _check(ts)
+
+
+def test_phases_leave_what_they_cannot_take(routes):
+    """Sums of 2^32 units, too many long-lived tensors, a long chain beside one: the general path."""
+    rng = np.random.default_rng(8)
+    ts = [_small(rng) for _ in range(36)]
+    ok = lambda: _trace(rng, 1200, 1300, 0.0, 64, 1 << 10)
+    for k, wide, longs, link in ((0, 0, 0, False), (1, 1, 0, False), (2, 0, 768, False), (3, 0, 769, False), (4, 0, 0, True),
+                                 (5, 0, 1, True)):
+        T, a, f, s = ok()
+        if link:
+            a, f = np.minimum(np.arange(len(a)), T - 3), np.minimum(np.arange(len(a)) + 2, T)
+        a[-1], f[-1] = 0, 2 if link and not longs else T  # held together by it
+        if longs > 1:
+            a[:longs - 1] = rng.integers(0, 300, longs - 1)
+            f[:longs - 1] = a[:longs - 1] + rng.integers(33, 800, longs - 1)
+            a[longs - 1:-1] = rng.integers(900, T - 5, len(a) - longs)
+            f[longs - 1:-1] = a[longs - 1:-1] + 1
+        if wide:
+            s[0] = (1 << 40) + 1
+        ts[k] = (T, a, f, s)
+    ts = tg.from_arrays(ts)
+    size, _, _ = _plans(ts, routes)
+    assert size == {"first": 30, "phases": 3, "general": 3}
+    _check(ts)
+
