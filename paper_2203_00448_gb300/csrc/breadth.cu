@@ -34,7 +34,9 @@ namespace mp {
 
 namespace {
 
-constexpr int32_t kBDeferred = -2;  // status of a trace left by k_breadth_comp to k_breadth_rest
+constexpr int32_t kBDeferred = -2;  // status of a trace left by k_breadth_comp: in phases, or tensor by tensor
+constexpr int32_t kBTensor = -3;    // ... tensor by tensor
+__device__ __forceinline__ bool left_over(int32_t status) { return status == kBDeferred || status == kBTensor; }
 
 // Per-trace working set: the breadth of the operator at each step; per tensor
 // (by id) its operator's breadth and step, (alloc, free), size and offset; the priority order; the
@@ -322,7 +324,17 @@ __device__ int32_t block_excl_max_i32(int32_t v, int32_t* red) {
 constexpr int32_t kBThreadComp = 8;
 constexpr int32_t kBWarpComp = 32;
 constexpr int32_t kBBigComps = 64;  // components of more than kBWarpComp members a trace may have here
-constexpr int32_t kBBigComp = 64;   // the most members of one, where the rest can be placed in phases
+constexpr int32_t kBBigComp = 64;   // the most members of one, where the trace can be placed in phases ...
+constexpr int32_t kBMidComp = 128;  // ... and where no trace of a very large batch has more tensors (comp_rule)
+constexpr int32_t kBLongLife = 32;  // lives above this many steps are long
+
+// Which traces with large components the component kernel leaves to the phases:
+// those with one of more than `comp` members, or whose components it cannot place
+// itself; but none that has `dense` or more short-lived tensors live at a step and
+// no long-lived ones.
+struct CompRule {
+    int32_t comp, dense;
+};
 
 // A tensor in alloc-step order with the keys of the breadth order.
 struct BRec {
@@ -488,13 +500,13 @@ __device__ void place_comp_warp(const BRec* __restrict__ R, int64_t* __restrict_
 
 __global__ void __launch_bounds__(kBreadthThreads)
 k_breadth_comp(mp_batch bt, int32_t policy, int64_t* __restrict__ offsets, int64_t* __restrict__ plan_peak,
-               int32_t* __restrict__ status, bool in_phases) {
+               int32_t* __restrict__ status, CompRule rule) {
     // once every CTA of this grid runs, those of k_breadth_rest may take what
     // room is left; they wait for this grid to finish
     asm volatile("griddepcontrol.launch_dependents;");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int64_t red[72];
-    __shared__ int32_t s_bad, s_defer, s_nt, s_nw, s_nb, s_cnt, s_bin[kBThreadComp - 1], s_base[kBThreadComp];
+    __shared__ int32_t s_bad, s_defer, s_nt, s_nw, s_nb, s_cnt, s_mid, s_lives, s_bin[kBThreadComp - 1], s_base[kBThreadComp];
     __shared__ int32_t s_mbase[kBThreadComp];    // the thread tier's members, by size class
     __shared__ uint32_t s_magic[kBThreadComp - 1];  // ceil(2^32 / c) of each size class
     __shared__ int32_t s_big[kBBigComps];
@@ -529,7 +541,7 @@ k_breadth_comp(mp_batch bt, int32_t policy, int64_t* __restrict__ offsets, int64
     }
     for (int32_t w = tid; w < nwords; w += nthr) SB[w] = 0;
     if (tid == 0) {
-        s_bad = s_defer = s_nt = s_nw = s_nb = 0;
+        s_bad = s_defer = s_nt = s_nw = s_nb = s_mid = s_lives = 0;
         s_hi = s_lo = 0;
     }
     if (tid < kBThreadComp - 1) s_bin[tid] = 0;
@@ -610,14 +622,27 @@ k_breadth_comp(mp_batch bt, int32_t policy, int64_t* __restrict__ offsets, int64
             LST[n - 1 - atomicAdd(&s_nw, 1)] = p * 64 + c;
         } else {  // the CTA tier, while its scratch holds the component
             const int32_t at = atomicAdd(&s_nb, 1);
-            if (at < kBBigComps && big_fits(c, T) && !(in_phases && c > kBBigComp)) s_big[at] = p;
+            if (at < kBBigComps && big_fits(c, T)) s_big[at] = p;
             else s_defer = 1;
+            if (c > rule.comp) s_mid = 1;
         }
     }
     __syncthreads();
-    if (s_defer) {  // too many large components, or one too large: another kernel places this trace
-        if (tid == 0) status[b] = kBDeferred;
-        return;
+    if (s_defer | s_mid) {  // (the same for every thread)
+        int32_t lives = 0;
+        bool any_long = false;
+        for (int32_t k = tid; k < n; k += nthr) {
+            const int32_t life = R[k].f - R[k].a;
+            any_long |= life > kBLongLife;
+            lives += life <= kBLongLife ? life : 0;
+        }
+        lives = __reduce_add_sync(0xffffffffu, lives);
+        if ((tid & 31) == 0) atomicAdd(&s_lives, lives);
+        const bool dense = !__syncthreads_or(any_long) && (int64_t)s_lives >= (int64_t)rule.dense * T;
+        if (s_defer || !dense) {
+            if (tid == 0) status[b] = dense ? kBTensor : kBDeferred;
+            return;
+        }
     }
     test_route(kRouteBreadthComp);
     if (tid == 0) {  // thread-tier components in descending size: bin starts, then cursors; member counts
@@ -764,8 +789,9 @@ k_breadth_rest(mp_batch bt, int32_t policy, int64_t* __restrict__ offsets, int64
     for (int64_t k0 = 0; blockIdx.x + k0 * gridDim.x < bt.n_traces; k0 += 32) {
         if (threadIdx.x < 32) {
             const int64_t b = blockIdx.x + (k0 + threadIdx.x) * gridDim.x;
-            const unsigned m =
-                __ballot_sync(0xffffffffu, b < bt.n_traces && (!deferred_only || status[b] == kBDeferred));
+            bool mine = b < bt.n_traces;
+            if (mine && deferred_only) mine = by_tensor ? left_over(status[b]) : status[b] == kBDeferred;
+            const unsigned m = __ballot_sync(0xffffffffu, mine);
             if (threadIdx.x == 0) s_todo = m;
         }
         __syncthreads();
@@ -774,7 +800,7 @@ k_breadth_rest(mp_batch bt, int32_t policy, int64_t* __restrict__ offsets, int64
         for (; m; m &= m - 1) {
             const int b = (int)(blockIdx.x + (k0 + __ffs(m) - 1) * gridDim.x);
             bool done = false;
-            if (phase_smem > 0) {
+            if (phase_smem > 0 && !(deferred_only && status[b] == kBTensor)) {
                 const TraceView tv = load_trace(bt, b, false);
                 if (tv.st == MP_OK && phases::fits<true>(tv.n, tv.T, phase_smem)) {
                     phases::Out o = {};
@@ -794,57 +820,131 @@ k_breadth_rest(mp_batch bt, int32_t policy, int64_t* __restrict__ offsets, int64
     }
 }
 
+// The traces k_breadth_comp and k_breadth_rest deferred (or all of them), tensor
+// by tensor with small CTAs.
+template <bool kSmem>
+__global__ void __launch_bounds__(kBreadthThreads)
+k_breadth_tensor(mp_batch bt, int32_t policy, int64_t* __restrict__ offsets, int64_t* __restrict__ plan_peak,
+                 int32_t* __restrict__ status, unsigned char* __restrict__ ws, size_t ws_stride, bool deferred_only) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    __shared__ unsigned s_todo;  // as in k_breadth_rest
+    for (int64_t k0 = 0; blockIdx.x + k0 * gridDim.x < bt.n_traces; k0 += 32) {
+        if (threadIdx.x < 32) {
+            const int64_t b = blockIdx.x + (k0 + threadIdx.x) * gridDim.x;
+            const unsigned m = __ballot_sync(0xffffffffu, b < bt.n_traces && (!deferred_only || left_over(status[b])));
+            if (threadIdx.x == 0) s_todo = m;
+        }
+        __syncthreads();
+        unsigned m = s_todo;
+        __syncthreads();
+        for (; m; m &= m - 1) {
+            const int b = (int)(blockIdx.x + (k0 + __ffs(m) - 1) * gridDim.x);
+            test_route(kRouteBreadthTensor);
+            breadth_trace<kSmem>(b, bt, policy, offsets, plan_peak, status, ws, ws_stride);
+            __syncthreads();
+        }
+    }
+}
+
 bool breadth_comp_fits(const mp_batch& bt) {
     return BCompLayout(bt.max_tensors, bt.max_steps).total <= kSmemCeiling;
 }
 
-// One launch of k_breadth_rest: in phases, tensor by tensor, or both.
+// Geometry of k_breadth_rest.
+struct RestGeometry {
+    size_t smem;
+    int threads, resident;
+};
 template <bool kSmem>
-cudaError_t launch_rest_once(const mp_batch& bt, int32_t policy, int64_t* offsets, int64_t* plan_peak, int32_t* status,
-                             void* workspace, bool deferred_only, size_t phase_smem, bool by_tensor,
-                             cudaStream_t stream) {
-    const size_t data = BreadthLayout(bt.max_tensors, bt.max_steps).total;
-    size_t smem = kSmem && by_tensor ? data : 0;
-    smem = std::max(smem, phase_smem);
-    const void* fn = (const void*)k_breadth_rest<kSmem>;
-    int sms = 0, resident = 0;
-    cudaError_t e = sm_count(&sms);
+cudaError_t rest_geometry(const mp_batch& bt, size_t phase_smem, bool by_tensor, int sms, RestGeometry* g) {
+    g->smem = std::max(kSmem && by_tensor ? BreadthLayout(bt.max_tensors, bt.max_steps).total : 0, phase_smem);
     // more traces than SMs: half the threads, where an SM holds two of them
-    const int threads =
-        bt.n_traces > sms && smem <= kTwoPerSm ? kBreadthPhaseThreads / 2 : kBreadthPhaseThreads;
-    if (e == cudaSuccess) e = set_smem_limit(fn, smem);
-    if (e == cudaSuccess) e = max_resident_ctas(fn, threads, smem, &resident);
-    if (e != cudaSuccess) return e;
+    g->threads = bt.n_traces > sms && g->smem <= kTwoPerSm ? kBreadthPhaseThreads / 2 : kBreadthPhaseThreads;
+    const void* fn = (const void*)k_breadth_rest<kSmem>;
+    const cudaError_t e = set_smem_limit(fn, g->smem);
+    return e != cudaSuccess ? e : max_resident_ctas(fn, g->threads, g->smem, &g->resident);
+}
+
+// The component kernel places large components tensor by tensor with its 128
+// threads, nine traces and more an SM, and k_breadth_tensor those it has no scratch
+// for; the phases hold two.  While they hold the whole batch at once they are the
+// faster ones (300 chains of 374 tensors 0.09 ms, 0.89 by components), except for
+// very dense traces (300 of 1,000 tensors over 10 steps: 34.2 and 30.0 ms).  In
+// larger batches they still are for chains (4,096: 1.00 and 1.94 ms), but not for
+// traces with more than a few tensors live at a step (2,048 of 512 tensors over 100
+// steps: 2.72 and 1.72 ms), nor, in very large ones, for traces little over the warp
+// tier (4,096 chains of 94: 0.49 and 0.28 ms, best fit 0.55 and 0.41; 1,024:
+// 0.14 and 0.13, 0.16 and 0.19).
+CompRule comp_rule(const mp_batch& bt, int32_t policy, size_t phase_smem, int sms) {
+    if (phase_smem == 0) return {INT32_MAX, 0};  // (what is left goes tensor by tensor either way)
+    if (bt.n_traces <= (phase_smem <= kTwoPerSm ? 2 * sms : sms)) return {kBBigComp, 100};
+    if (bt.max_tensors <= kBMidComp && bt.n_traces > (policy == MP_FIT_FIRST ? 6 : 12) * sms) return {kBMidComp, 0};
+    return {kBBigComp, 8};
+}
+
+// A launch that waits in the kernel for the one before it in this call.
+template <typename... Params, typename... Args>
+cudaError_t launch_next(void (*kernel)(Params...), int grid, int threads, size_t smem, cudaStream_t stream, bool follows,
+                        Args... args) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)std::min(bt.n_traces, resident));
+    cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = deferred_only ? 1 : 0;  // (it follows a kernel of this call)
+    attr[0].val.programmaticStreamSerializationAllowed = follows ? 1 : 0;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_breadth_rest<kSmem>, bt, policy, offsets, plan_peak, status,
-                              static_cast<unsigned char*>(workspace), data, deferred_only, (uint32_t)phase_smem,
-                              by_tensor);
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-// Both ways in one launch where that leaves room for two CTAs an SM, else one
-// launch each: 256 traces of 2,000 tensors take 0.32 ms so, and 0.45 ms with
-// the 160 KB that placing one of them tensor by tensor would need.
+// What k_breadth_comp leaves (comp; otherwise all traces).  Both ways in one launch
+// where that holds the batch at once and what places tensor by tensor wants no
+// shared memory that the phases do not leave it -- 256 traces of 2,000 tensors take
+// 0.32 ms so, and 0.45 ms with the 160 KB that placing one of them tensor by tensor
+// would need --, nor, with its data in the workspace, the L1 cache instead (40 chains
+// and a trace of 5,000 tensors: 15.6 ms in one launch, 5.7 apart).  A batch
+// that is more than one wave of its CTAs is placed tensor by tensor with small ones
+// (1,000 traces of 1,500 tensors, none of them for the phases: 22.7 ms with the
+// phases' registers, 17.1 so).
 template <bool kSmem>
 cudaError_t launch_rest(const mp_batch& bt, int32_t policy, int64_t* offsets, int64_t* plan_peak, int32_t* status,
-                        void* workspace, bool deferred_only, size_t phase_smem, cudaStream_t stream) {
+                        void* workspace, bool comp, size_t phase_smem, int sms, cudaStream_t stream) {
     const size_t data = BreadthLayout(bt.max_tensors, bt.max_steps).total;
-    if (kSmem && phase_smem > 0 && data > std::max(phase_smem, kTwoPerSm)) {
-        const cudaError_t e = launch_rest_once<kSmem>(bt, policy, offsets, plan_peak, status, workspace, deferred_only,
-                                                      phase_smem, false, stream);
+    unsigned char* ws = static_cast<unsigned char*>(workspace);
+    bool deferred_only = comp;
+    RestGeometry g;
+    // (a CTA that an SM takes on while the phases still run there gets the little L1
+    // cache that they leave, for as long as it runs: not where its data are in the
+    // workspace)
+    auto rest = [&](size_t phases_with, bool by_tensor) {
+        return launch_next(k_breadth_rest<kSmem>, std::min(bt.n_traces, g.resident), g.threads, g.smem, stream,
+                           deferred_only && (kSmem || phases_with > 0), bt, policy, offsets, plan_peak, status, ws,
+                           data, deferred_only, (uint32_t)phases_with, by_tensor);
+    };
+    cudaError_t e = rest_geometry<kSmem>(bt, phase_smem, true, sms, &g);
+    if (e != cudaSuccess) return e;
+    if (phase_smem > 0) {
+        if (bt.n_traces <= g.resident && kSmem && data <= std::max(phase_smem, kTwoPerSm)) return rest(phase_smem, true);
+        e = rest_geometry<kSmem>(bt, phase_smem, false, sms, &g);
+        if (e == cudaSuccess) e = rest(phase_smem, false);
+        deferred_only = true;
+        if (e == cudaSuccess) e = rest_geometry<kSmem>(bt, 0, true, sms, &g);
         if (e != cudaSuccess) return e;
-        return launch_rest_once<kSmem>(bt, policy, offsets, plan_peak, status, workspace, true, 0, true, stream);
     }
-    return launch_rest_once<kSmem>(bt, policy, offsets, plan_peak, status, workspace, deferred_only, phase_smem, true,
-                                   stream);
+    if (bt.n_traces <= g.resident) return rest(0, true);
+    const size_t smem = kSmem ? data : 0;
+    int resident = 0;
+    e = set_smem_limit((const void*)k_breadth_tensor<kSmem>, smem);
+    if (e == cudaSuccess)
+        e = max_resident_ctas((const void*)k_breadth_tensor<kSmem>, kBreadthThreads, smem, &resident);
+    if (e != cudaSuccess) return e;
+    // (two waves of CTAs, so that the second evens the first out: a whole CTA for every
+    // trace that has nothing to do costs 1.5 us with 4,096 of them)
+    return launch_next(k_breadth_tensor<kSmem>, (int)std::min<int64_t>(bt.n_traces, 2 * (int64_t)resident),
+                       kBreadthThreads, smem, stream, deferred_only && kSmem, bt, policy, offsets, plan_peak, status,
+                       ws, data, deferred_only);
 }
 
 }  // namespace
@@ -867,13 +967,14 @@ cudaError_t launch_breadth(const mp_batch& bt, int32_t policy, int64_t* offsets,
         e = set_smem_limit((const void*)k_breadth_comp, cbytes);
         if (e != cudaSuccess) return e;
         k_breadth_comp<<<(unsigned)bt.n_traces, kBreadthThreads, cbytes, stream>>>(bt, policy, offsets, plan_peak,
-                                                                                  status, phase_smem > 0);
+                                                                                  status,
+                                                                                  comp_rule(bt, policy, phase_smem, sms));
         e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
+        if (e != cudaSuccess || bt.max_tensors <= kBWarpComp) return e;  // no component is too large for it
     }
     return breadth_fits_smem(bt)
-               ? launch_rest<true>(bt, policy, offsets, plan_peak, status, workspace, comp, phase_smem, stream)
-               : launch_rest<false>(bt, policy, offsets, plan_peak, status, workspace, comp, phase_smem, stream);
+               ? launch_rest<true>(bt, policy, offsets, plan_peak, status, workspace, comp, phase_smem, sms, stream)
+               : launch_rest<false>(bt, policy, offsets, plan_peak, status, workspace, comp, phase_smem, sms, stream);
 }
 
 }  // namespace mp

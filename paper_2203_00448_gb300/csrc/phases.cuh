@@ -141,7 +141,8 @@ __host__ __device__ bool fits(int32_t n, int32_t T, size_t smem) {
 // for the longest; where that is too much, as in a batch of ordinary traces with
 // a very long one among them, what leaves an SM as many CTAs as the batch can
 // use, and the traces it holds are placed here (600 chains of 374 tensors and a
-// trace of 2,000 over 20,000 steps: MIXEDUS); 0 if few would be.
+// trace of 2,000 over 20,000 steps: 1.32 ms by the general path, 0.46 so); 0 if few
+// would be.
 template <bool kBreadth>
 size_t smem_bytes(const mp_batch& bt, int sms) {
     if (fits<kBreadth>(bt.max_tensors, bt.max_steps, kSmemCeiling))

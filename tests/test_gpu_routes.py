@@ -18,7 +18,7 @@ def _linked(rng, n, sizes=64, life=3):
 
 
 def _small(rng):
-    return _trace(rng, 40, 40, 0.0, 64, 1 << 14)
+    return _trace(rng, 30, 40, 0.0, 64, 1 << 14)
 
 
 def _plans(ts, routes):
@@ -150,3 +150,51 @@ def test_phases_leave_what_they_cannot_take(routes):
     assert size == {"first": 30, "phases": 3, "general": 3}
     _check(ts)
 
+
+@pytest.mark.parametrize("traces,n,first,best", ((34, 64, "comp", "comp"), (34, 65, "phases", "phases"),
+                                                 (913, 128, "tensor", "phases"), (913, 129, "phases", "phases"),
+                                                 (1825, 128, "tensor", "tensor")))
+def test_breadth_chains(routes, traces, n, first, best):
+    rng = np.random.default_rng(n + traces)
+    ts = [_small(rng) for _ in range(traces)]
+    for k in (0, traces - 1):
+        ts[k] = _linked(rng, n)
+    if n == 64:
+        ts[0] = (2 * n + ts[0][0], *ts[0][1:])  # steps, the component kernel's scratch
+        ts[traces - 1] = ts[0]
+    ts = tg.from_arrays(ts)
+    got = _plans(ts, routes)[1:]
+    assert got == tuple({"breadth-comp": traces} if r == "comp" else {"breadth-comp": traces - 2, "breadth-" + r: 2}
+                        for r in (first, best))
+    _check(ts)
+
+
+# tensors of a step: on either side of the lines for a batch that the phases hold at once, and for a larger one
+@pytest.mark.parametrize("traces,per_step,route", ((34, 101, "phases"), (34, 102, "tensor"), (310, 7, "phases"),
+                                                   (310, 8, "tensor")))
+def test_breadth_dense(routes, traces, per_step, route):
+    rng = np.random.default_rng(per_step + traces)
+    ts = [_small(rng) for _ in range(traces)]
+    a = np.repeat(np.arange(40), per_step)
+    f = a + 1
+    f[::per_step] += 1  # links its step to the next
+    ts[5] = (41, a, f, rng.integers(1, 1 << 10, len(a)) * 64)
+    ts = tg.from_arrays(ts)
+    got = _plans(ts, routes)[1:]
+    assert got[0] == got[1] == {"breadth-comp": traces - 1, "breadth-" + route: 1}
+    _check(ts)
+
+
+def test_breadth_tensor_by_tensor_with_small_ctas(routes):
+    """More traces than the phases' launch holds at once, some of which it refuses."""
+    rng = np.random.default_rng(3)
+    ts = [_small(rng) for _ in range(400)]
+    for k in (0, 199, 399):
+        T, a, f, s = _trace(rng, 300, 400, 0.05, 1, 1 << 10, full_span=True)
+        s[0] = (1 << 40) + 1
+        ts[k] = (T, a, f, s)
+    ts[7] = _trace(rng, 300, 400, 0.05, 1, 1 << 10, full_span=True)
+    ts = tg.from_arrays(ts)
+    got = _plans(ts, routes)[1:]
+    assert got[0] == got[1] == {"breadth-comp": 396, "breadth-phases": 1, "breadth-tensor": 3}
+    _check(ts)
