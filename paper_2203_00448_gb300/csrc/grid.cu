@@ -82,6 +82,7 @@ constexpr size_t kGridSmem = kRegionBytes + kCacheBytes;
 constexpr int32_t kLongPredPairs = 9216;
 constexpr int32_t kLongSuccs = (int32_t)((kRegionBytes - (size_t)kLongPredPairs * 16) / 4);
 constexpr int32_t kRegionPairs = kLongPredPairs;  // CTA-item pairs beyond this go to the overflow buffer
+static_assert(kRegionPairs == kFlowPairs, "what the estimates count with");
 constexpr int32_t kWarpBytes = (int32_t)(kRegionBytes / 16);
 constexpr int32_t kWarpSortPairs = 512;
 constexpr int32_t kWarpPairs = 448;  // predecessors a warp holds while it places a short tensor
@@ -392,8 +393,9 @@ __global__ void __launch_bounds__(kPrepThreads) k_grid_prep(mp_batch bt, GridOut
         // (a test that holds a tensor back means the dataflow's queues)
         const bool narrow = (((s_hi << 32) + s_lo) >> ti->shift) <= 0xffffffffull;
         if (w.p_af != nullptr && w.hold < 0 && narrow) {
-            const int pays = choose_phases(n, nlong, (int64_t)s_long, (int64_t)s_short, T, out.policy);
-            if (pays >= 0) atomicAdd(pays > 0 ? &w.ctl->votes : &w.ctl->neutral, 1);
+            const int64_t room = chain_room(n, nlong, (int64_t)s_long, (int64_t)s_short, T, out.policy);
+            ti->room = (int32_t)(room < INT32_MAX ? room : INT32_MAX);
+            if (room >= 0) atomicAdd(n > 1024 ? &w.ctl->votes : &w.ctl->neutral, 1);
         }
     }
 }
@@ -1110,8 +1112,7 @@ k_grid_flow(mp_batch bt, int32_t policy, GridWs w, int32_t long_ctas) {
     GridCtl* ctl = w.ctl;
     if (in_phases(ctl)) {
         int32_t rounds = 0;
-        far_prepare(bt, w, smem_raw, red, [&]() { return grid_barrier(ctl, ++rounds, test_absent(w)); });
-        return;
+        if (far_prepare(bt, w, smem_raw, red, [&]() { return grid_barrier(ctl, ++rounds, test_absent(w)); })) return;
     }
 
     if (blockIdx.x == 0)

@@ -23,6 +23,8 @@ constexpr int32_t kFarMaxTensors = 32767;  // positions and ranks are 16-bit wor
 constexpr int32_t kPer = 4;                // buckets of addresses per thread, while a long-lived tensor is placed
 constexpr int32_t kBuckets = kPer * kFarThreads;
 constexpr int32_t kSegments = kBuckets / 8;  // address ranges looked at more closely at a time
+constexpr int32_t kFlowPairs = 9216;       // predecessors of a long-lived tensor that the dataflow's shared memory holds
+constexpr int32_t kLeastRoom = 128;        // no more than it costs to find out how long the chains are
 constexpr int32_t kEdges = 1024;           // positions before a window's core whose overlap is kept as bits
 
 // Shared memory of k_far_place for n tensors, nl of them long-lived.
@@ -44,30 +46,48 @@ struct FarLayout {
 };
 constexpr size_t kFarSmem = 225 * 1024;  // of the 227 KB a CTA may have; the rest is static
 
-// Whether a checked trace can be placed in phases: 1 if one SM is expected to
-// place it sooner than the whole GPU's dataflow, 0 if it can be but matters
-// little (a small trace in a batch of large ones), -1 if not.  Estimates in us.
-// One SM pays for every long-lived tensor with the run before it, more the
-// larger the windows (FIRST: 12 us each with 20,000 tensors, 7 with 2,000; BEST
-// looks at every gap: 43 and 14).  The dataflow pays for its long-lived tensors
-// one after the other where they are live together (`together` of them on
-// average), each the slower the more they are.  Measured, dataflow / phases, ms:
-// long tails of 20,000, 5,000 and 1,500 tensors 25.2 / 12.0, 3.1 / 2.3 and 0.89 /
-// 0.76 (FIRST), 31.4 / 42.9, 3.6 / 4.7 and 1.12 / 1.17 (BEST); seq2seq, 2,000
-// tensors with 40 that span the trace, 1.02 / 0.53 and 1.08 / 0.57.  Without
-// long-lived tensors, or with more neighbours than are listed per short one,
-// the dataflow's width wins.
-__host__ __device__ inline int choose_phases(int64_t n, int64_t nlong, int64_t long_steps, int64_t short_steps,
-                                             int64_t T, int32_t policy) {
+// The longest chain (alloc-order positions from the first to the last member of a
+// component of short lifetimes) with which one SM is expected to place a checked
+// trace in phases sooner than the whole GPU's dataflow would; -1 if it cannot or
+// is not whatever the chains, INT32_MAX if they do not matter (a small trace in a
+// batch of large ones).  Estimates, in us, of what was measured over traces of
+// 2,000 to 20,000 tensors, 2 to 6 a step, with long-lived ones that span the trace
+// or a part of it (dataflow / phases, ms: 20,000, 1,000 of them long, 2 a step 30.4 /
+// 12.0 FIRST, 33.8 / 42.9 BEST, 6 a step 32.8 / 44.1 FIRST; 2,000, 4 a step 1.54 /
+// 1.74 and 1.94 / 4.56; 20,000 in one chain, 10 that span it 2.2 / 6.8, 100 that do
+// 33.6 / 5.3):
+//   - the dataflow places long-lived tensors that are live together one after
+//     another, at most some 2.7 times as many in a row as are live on average,
+//     each after looking at the tensors allocated during its life, several times
+//     as slowly where these do not fit its shared memory;
+//   - one SM pays for every long-lived tensor with the run before it; BEST looks at
+//     every gap, of which long-lived tensors that overlap in part leave more; and
+//     for the short-lived ones where their number is large;
+//   - one warp walks a chain, member by member: 0.9 us each, more where many are
+//     live at a step.
+// Without long-lived tensors, or with more neighbours than are listed per short
+// one, the dataflow's width wins.
+__host__ __device__ inline int64_t chain_room(int64_t n, int64_t nlong, int64_t long_steps, int64_t short_steps,
+                                              int64_t T, int32_t policy) {
     if (n > kFarMaxTensors || nlong > kFarMaxLong || T > 65535 || 2 * short_steps > (int64_t)phases::kNear * T)
         return -1;
     if (FarLayout((int32_t)n, (int32_t)nlong).total > kFarSmem) return -1;
-    if (n <= 1024) return 0;
+    if (n <= 1024) return INT32_MAX;
     if (nlong == 0) return -1;
-    const int64_t together = long_steps / T;
-    const int64_t phased = 150 + nlong * (policy == MP_FIT_FIRST ? 6 + n / 3300 : 10 + n / 600);
-    const int64_t flow = 45 * together + 3 * together * together / 10;
-    return phased <= flow ? 1 : -1;
+    const bool first = policy == MP_FIT_FIRST;
+    const int64_t most = 27 * long_steps / (10 * T), hops = most < nlong ? most : nlong;
+    const int64_t seen = n * long_steps / (T * nlong);  // tensors allocated during a long-lived one's life
+    int64_t flow = hops * (1950 + seen) / 130;
+    if (!first) flow = flow * 115 / 100;
+    if (seen > kFlowPairs) flow *= first ? 2 : 4;
+    int64_t phased = 150 + n * n / 120000;
+    if (first) phased += nlong * (5000 + n / 5) / 1000;
+    else phased += (nlong * (7000 + n * 2 / 3) + (nlong - long_steps / T) * (3000 + n * 10 / 9)) / 1000;
+    if (phased > flow) return -1;
+    const int64_t live = 10 * short_steps / T;  // tenths
+    const int64_t member = first ? 930 + (live > 90 ? 11 * (live - 90) : 0) : 400 + 29 * live;  // ns
+    const int64_t room = (flow - phased) * 1000 / member;
+    return room < kLeastRoom ? -1 : room;
 }
 
 // Queues and counters shared by the whole grid.
@@ -78,16 +98,18 @@ struct GridCtl {
     int32_t placed;          // tensors placed so far
     int32_t fail;            // a CTA gave up waiting
     int32_t checked;         // traces that passed their checks ...
-    int32_t votes, neutral;  // ... for which phases pay, and which fit them (choose_phases)
+    int32_t votes, neutral;  // ... for which phases may pay, and which fit them (chain_room)
+    int32_t against;         // ... whose chains turned out too long for them
     int32_t arrived;         // CTAs that reached the grid's barriers, all told
     int32_t finished;        // CTAs of k_grid_finish that are done
 };
 
 // Whether the batch's traces are placed by one CTA each in phases
 // (grid_phases.cuh) instead of by the dataflow: all of them or none, since the
-// two would run one after the other (once k_grid_prep has finished).
+// two would run one after the other.  Once k_grid_prep has finished this says
+// whether it may be; once the chains are known (far_comps) whether it is.
 __device__ __forceinline__ bool in_phases(const GridCtl* ctl) {
-    return ctl->votes > 0 && ctl->votes + ctl->neutral == ctl->checked;
+    return ctl->votes > 0 && ctl->votes + ctl->neutral == ctl->checked && *(const volatile int32_t*)&ctl->against == 0;
 }
 
 // Per-trace state.
@@ -99,6 +121,7 @@ struct TraceInfo {
     int32_t ok;               // 1 once the trace passed its checks
     int32_t incomplete;       // a tensor was left unplaced
     int32_t shift;            // every size is a multiple of 1 << shift (a unit)
+    int32_t room;             // the longest chain for which phases pay (chain_room)
 };
 
 // A tensor in alloc-step order (16 bytes: one vector load).

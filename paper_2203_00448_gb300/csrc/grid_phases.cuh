@@ -13,7 +13,8 @@
 // first:
 //
 //   far_sort   stable alloc order (alloc step, then id) of every tensor;
-//   far_comps  components of short lifetimes, a CTA per trace;
+//   far_comps  components of short lifetimes, a CTA per trace; with chains too
+//              long for one SM the batch goes back to the dataflow;
 //   far_rank   priority ranks, by counting (every pair of tensors once);
 //   far_link   records by rank: windows, chain links, neighbour lists;
 //   far_place  one CTA per trace.
@@ -24,7 +25,7 @@
 //
 // A trace is placed in phases when its sizes sum below 2^32 units, it fits the
 // shared memory, and one SM is likely to beat the dataflow (grid.cuh:
-// choose_phases, which k_grid_prep asks).
+// chain_room, which k_grid_prep asks).
 #pragma once
 
 #include "grid.cuh"
@@ -75,6 +76,7 @@ __device__ __forceinline__ void far_comps(const GridWs& w, int32_t b, uint32_t* 
     }
     start = phases::block_excl_max(start, red, &tot);
     run = before;
+    int32_t longest = 0;
     for (int32_t q = q0; q < q1; ++q) {
         const uint32_t af = AF[q];
         if (life(af) > kLong) {
@@ -84,7 +86,9 @@ __device__ __forceinline__ void far_comps(const GridWs& w, int32_t b, uint32_t* 
         if (run <= (af & 0xffffu)) start = (uint32_t)q + 1;
         run = max(run, af >> 16);
         w.p_cs[base + q] = start;
+        longest = max(longest, q + 1 - (int32_t)start + 1);
     }
+    if (__syncthreads_or(longest > w.ti[b].room) && t == 0) atomicAdd(&w.ctl->against, 1);
 }
 
 // Ranks by (size descending, position): every tensor against a slice of the
@@ -482,12 +486,14 @@ __device__ __forceinline__ void far_place(const GridWs& w, int32_t b, int32_t po
 }
 
 // Everything before far_place, by the whole cooperative grid: `sync` is a
-// barrier over it, false when its bounded wait ran out.
+// barrier over it, false when its bounded wait ran out.  Returns false if the
+// batch's chains leave it to the dataflow after all (some 20 us for a trace of
+// 2,000 tensors, 40 for 20,000).
 template <typename Sync>
-__device__ __forceinline__ void far_prepare(const mp_batch& bt, const GridWs& w, unsigned char* smem, int64_t* red,
+__device__ __forceinline__ bool far_prepare(const mp_batch& bt, const GridWs& w, unsigned char* smem, int64_t* red,
                                             Sync&& sync) {
     far_sort(bt, w);
-    if (!sync()) return;
+    if (!sync()) return true;
     int32_t item = 0;
     for (int32_t b = 0; b < bt.n_traces; ++b) {
         if (!w.ti[b].ok) continue;
@@ -498,9 +504,10 @@ __device__ __forceinline__ void far_prepare(const mp_batch& bt, const GridWs& w,
                 if (item % (int32_t)gridDim.x == (int32_t)blockIdx.x)
                     far_rank_tile(w, b, i0, j0, reinterpret_cast<uint64_t*>(smem));
     }
-    if (!sync()) return;
+    if (!sync()) return true;
+    if (!in_phases(w.ctl)) return false;
     far_link(bt, w);
-    __syncthreads();
+    return true;
 }
 
 }  // namespace grid

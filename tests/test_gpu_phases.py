@@ -124,9 +124,10 @@ def _far_trace(rng, n, T, kind):
         s = rng.choice([64, 4096, 1 << 20], n)
     elif kind == "crowded-steps":  # over kEdges tensors just before a long one's start, chains past kNear neighbours
         a[: 1500] = rng.integers(10, 14, 1500)
-        f = a + rng.integers(1, 6, n)
+        f = a + rng.integers(1, 9, n)
         f[:4] = a[:4] + 60
         a[4:8], f[4:8] = 16, T
+        a[8:308], f[8:308] = 0, T  # enough that phases pay
     elif kind == "wide-sums":  # past 2^32 units: the dataflow
         s[0], s[1] = (1 << 35) + 1, 1
     elif kind == "short-only":

@@ -6,7 +6,7 @@ import pytest
 
 import tracegen as tg
 
-from tests.test_gpu_phases import _check, _trace
+from tests.test_gpu_phases import _check, _far_trace, _trace
 
 pytestmark = pytest.mark.gpu
 
@@ -198,3 +198,37 @@ def test_breadth_tensor_by_tensor_with_small_ctas(routes):
     got = _plans(ts, routes)[1:]
     assert got[0] == got[1] == {"breadth-comp": 396, "breadth-phases": 1, "breadth-tensor": 3}
     _check(ts)
+
+
+def _spanned(rng, n, longs):
+    """One chain of n tensors, `longs` of which span it instead."""
+    T, a, f, s = _linked(rng, n, 1 << 12)
+    far = rng.permutation(n)[:longs]
+    a[far], f[far] = 0, T
+    return T, a, f, s
+
+
+@pytest.mark.parametrize("kind,n,first,best", (("long-tail", 5000, "phases", "flow"), ("full-span", 6001, "phases", "phases"),
+                                               ("crowded-steps", 7000, "phases", "phases"), ("wide-sums", 4500, "flow", "flow"),
+                                               ("short-only", 5000, "flow", "flow"), ("all-long", 4200, "flow", "flow"),
+                                               ("chain-10", 2000, "flow", "flow"), ("chain-30", 2000, "phases", "phases"),
+                                               ("dense", 2000, "flow", "flow")))
+def test_large_traces(routes, kind, n, first, best):
+    import paper_2203_00448_gb300 as mp
+
+    rng = np.random.default_rng(n + len(kind))
+    if kind.startswith("chain"):
+        t = _spanned(rng, n, int(kind[6:]))
+    elif kind == "dense":  # few gaps between the chains of short-lived tensors: one warp would walk nearly all
+        t = _far_trace(rng, n, n // 5, "long-tail")
+    else:
+        t = _far_trace(rng, n, n // 2 + 100, kind)
+    empty = np.zeros(0, np.int64)
+    ts = tg.from_arrays([t, (5, empty, empty, empty)])
+    db = mp.DeviceBatch.from_host(ts, "cuda")
+    for policy, route in (("first", first), ("best", best)):
+        for fn in (mp.plan_and_validate, mp.plan_greedy_by_size):
+            fn(db, policy)
+            assert routes() == {"grid-" + route: 2}, policy
+    if n <= 5000:
+        _check(ts)
