@@ -79,8 +79,9 @@ def build(force: bool = False, verbose: bool = False, extra_flags=None) -> str:
 
 TEST_HOOKS_DIR = os.path.join(BUILD_DIR, "test_hooks")
 TEST_HOOKS_LIB = os.path.join(TEST_HOOKS_DIR, "libmemplan_test_hooks.so")
-# Test builds: the entry point mp_test_plan_hold, and bounds on the planner's
-# waits of about 8 ms instead of about a second.
+# Test builds: the entry points mp_test_*, which hold a tensor back or say which
+# kernels placed the traces, and bounds on the planner's waits of about 8 ms instead
+# of about a second.
 TEST_HOOKS_FLAGS = ["-DMP_TEST_HOOKS", "-DMP_TEST_SPIN_CYCLES=(1ll<<24)", "-DMP_TEST_GRID_SPIN_CYCLES=(1ll<<24)"]
 
 

@@ -10,20 +10,21 @@
 // operator's step (the earlier on ties), then size descending, alloc step
 // ascending, id ascending.
 //
-// GPU form: one CTA per trace, in two kernels.  k_breadth_comp places every
-// trace whose working set fits in shared memory by lifetime components (see its
-// comment below): a thread, a warp or the whole CTA per component.  The traces
-// it leaves (a component past kBBigComp tensors, or too many of its large ones)
-// go to k_breadth_rest, which places a trace's short-lived tensors by chains and
-// its long-lived ones by the whole CTA over a list sorted by offset
-// (phases.cuh): 256 traces of 2,000 tensors take 0.32 ms instead of 38.5 ms.
-// What that path does not take (sizes past 2^32 units, too many long-lived
-// tensors, traces past its limits) is placed there tensor by tensor
-// (breadth_trace): the breadths (two integer atomics per tensor, order-
-// independent), each tensor's wider operator, an in-place odd-even merge sort of
-// the ids by that order, then for each tensor all warps gather the placed
-// tensors whose lifetimes overlap it (one shared counter update per warp) and
-// warp 0 runs the gap search with warp reductions.
+// GPU form: one CTA per trace.  k_breadth_comp places every trace whose working
+// set fits in shared memory by lifetime components (see its comment below): a
+// thread, a warp or the whole CTA per component.  Of the traces it leaves (a
+// component past kBBigComp tensors, or too large or too many for it)
+//   - k_breadth_rest places short-lived tensors by chains and long-lived ones by
+//     the whole CTA over a list sorted by offset (phases.cuh): 256 traces of 2,000
+//     tensors take 0.32 ms instead of 38.5 ms;
+//   - what that path does not take (sizes past 2^32 units, too many long-lived
+//     tensors, traces past its limits) or is no gain for (comp_rule) is placed
+//     tensor by tensor (breadth_trace), there or by k_breadth_tensor: the breadths
+//     (two integer atomics per tensor, order-independent), each tensor's wider
+//     operator, an in-place odd-even merge sort of the ids by that order, then for
+//     each tensor all warps gather the placed tensors whose lifetimes overlap it (one
+//     shared counter update per warp) and warp 0 runs the gap search with warp
+//     reductions.
 #include <algorithm>
 
 #include "common.cuh"
@@ -287,10 +288,10 @@ bool breadth_fits_smem(const mp_batch& bt) {
 // components (a run starts where no earlier tensor is still live), and places
 // each component in the breadth order -- one thread for up to kBThreadComp
 // members, one warp (a member per lane) for up to kBWarpComp, the whole CTA
-// beyond.  Traces with more than kBBigComps such large components, or one past
-// kBBigComp members or too large for the CTA tier's scratch, and batches whose
+// beyond.  Traces with more than kBBigComps such large components, or one that is
+// better placed in phases or too large for the CTA tier's scratch, and batches whose
 // working set does not fit in shared memory, are left to the other kernels
-// (status kBDeferred in between).
+// (status kBDeferred or kBTensor in between).
 
 // Exclusive prefix maximum (identity 0) of one non-negative value per thread
 // over the block; ends with a barrier.  red: >= 33 slots.

@@ -16,7 +16,7 @@ constexpr int kPeakThreads = 128;
 constexpr int kBumpThreads = 128;
 constexpr int kReplayThreads = 256;
 constexpr int kBreadthThreads = 128;
-constexpr int kBreadthPhaseThreads = 512;  // half of it when the batch has more traces than the GPU SMs
+constexpr int kBreadthPhaseThreads = 512;  // half of it in a batch of more traces than SMs, where an SM holds two CTAs
 constexpr int kPlanThreadsSmem = 128;    // one CTA per trace, data in shared memory
 constexpr int kPlanThreadsFew = 512;     // ... in a batch of few traces
 constexpr int kPlanThreadsGlobal = 1024; // one CTA per trace, data in the workspace

@@ -1,6 +1,6 @@
 // phases.cuh -- greedy placement of one trace by one CTA in phases, for traces
 // whose lifetimes link many tensors (components past the warp tier): the
-// deferred traces of greedy_by_size (plan.cu) and of greedy by breadth
+// deferred traces of greedy_by_size (plan.cuh) and of greedy by breadth
 // (breadth.cu).
 //
 // The sequential definition takes tensors in priority order and gives each a

@@ -55,9 +55,10 @@
 // tensor, so every offset, end and live-bytes value of a trace is at most the
 // sum of its sizes.  Each call therefore launches the kernel twice: first with
 // 32-bit byte arithmetic (W = uint32_t), which handles every trace of small
-// components whose sizes sum below 2^32 and marks the others deferred; then
-// with larger CTAs and 64-bit arithmetic (the phases count in units and stay
-// in 32 bits), which return at once unless a trace was deferred.
+// components, or of large ones that it walks, whose sizes sum below 2^32 and marks
+// the others deferred; then with larger CTAs and 64-bit arithmetic (the phases
+// count in units and stay in 32 bits), which return at once unless a trace was
+// deferred.
 //
 // Fused pass (mp_plan_and_validate): the difference array of the profile is
 // built while the inputs are first read, scanned and written out before the
@@ -1621,7 +1622,11 @@ __device__ __forceinline__ int32_t test_hold_position(int) { return -1; }
 
 // ------------------------------------------------------------- the kernel
 
-enum Tier { kTierNone, kTierWalk, kTierCta };  // what places components of more than kWarpComp tensors
+// What places components of more than kWarpComp tensors: the second launch; a warp
+// each (walk_tier); the CTA tier; the phases, or the CTA tier where they do not take
+// the trace.  (A batch that the phases cannot take gets a kernel without them: with
+// their code in it the CTA tier is slower, 310 chains of 2,000 steps 5.0 ms and 4.5.)
+enum Tier { kTierNone, kTierWalk, kTierCta, kTierPhases };
 
 // The whole path for trace b, by the whole CTA.
 template <typename I, typename W, bool kSmem, bool kFused, Tier kTier>
@@ -2111,7 +2116,7 @@ __device__ __forceinline__ bool plan_in_phases(const int b, const mp_batch& bt, 
 // 32-bit launch: one CTA per trace.  64-bit launch: a grid no larger than
 // what the GPU holds at once walks every trace and takes the ones the 32-bit
 // launch deferred (sizes summing to 2^32 or more, or a component the 32-bit
-// launch does not place), with larger CTAs for the CTA tier.
+// launch does not place), with larger CTAs for the phases and the CTA tier.
 template <typename I, typename W, bool kSmem, bool kFused, int kThreads, Tier kTier>
 __global__ void __launch_bounds__(kThreads, sizeof(W) == 8 || !kSmem ? 1 : kThreads == kPlanThreadsFew ? 2 : kPlanCtasSmem)
 k_plan(mp_batch bt, PlanOut out, unsigned char* __restrict__ ws, size_t data_stride, size_t buf_offset,
@@ -2140,9 +2145,9 @@ k_plan(mp_batch bt, PlanOut out, unsigned char* __restrict__ ws, size_t data_str
                 const int b = (int)(blockIdx.x + (k0 + __ffs(m) - 1) * gridDim.x);
                 m &= m - 1;
                 bool done = false;
-                if constexpr (sizeof(I) == 2) done = phase_smem > 0 && plan_in_phases<kFused>(b, bt, out, phase_smem);
+                if constexpr (kTier == kTierPhases) done = plan_in_phases<kFused>(b, bt, out, phase_smem);
                 if (!done)
-                    plan_trace<I, W, kSmem, kFused, kTier>(b, bt, out, ws, data_stride, buf_offset, buf_stride, rule);
+                    plan_trace<I, W, kSmem, kFused, kTierCta>(b, bt, out, ws, data_stride, buf_offset, buf_stride, rule);
                 __syncthreads();
             }
         }
@@ -2233,7 +2238,7 @@ cudaError_t launch_variant(const mp_batch& bt, const PlanGeometry& g, const Plan
         if (e != cudaSuccess) return e;
     }
     // for the traces that are placed in phases (0: none)
-    const size_t phase_smem = sizeof(W) == 8 && sizeof(I) == 2 ? phases::smem_bytes<false>(bt, sms) : 0;
+    const size_t phase_smem = kTier == kTierPhases ? phases::smem_bytes<false>(bt, sms) : 0;
     smem = std::max(smem, phase_smem);
     // more traces than SMs: half the threads, where an SM holds two of them
     if (phase_smem > 0 && bt.n_traces > sms && smem <= kTwoPerSm) threads /= 2;
@@ -2277,24 +2282,35 @@ cudaError_t launch_width(const mp_batch& bt, const PlanOut& out, unsigned char* 
     const PlanWorkspace pw = plan_workspace(bt);
     constexpr int kSmemThreads = sizeof(W) == 8 ? kPlanThreadsWide : kPlanThreadsSmem;
     constexpr int kGlobalThreads = sizeof(W) == 8 ? kPlanThreadsWide : kPlanThreadsGlobal;
+    int sms = 0;
+    const cudaError_t e = sm_count(&sms);
+    if (e != cudaSuccess) return e;
+    const bool phased = g.narrow && phases::smem_bytes<false>(bt, sms) > 0;
     if constexpr (sizeof(W) == 4) {
-        // traces of some length, too few to fill the GPU with 128 threads each:
-        // the latency of one CTA is what counts, and more threads shorten all
-        // but the placement of its longest component (301 ragged traces of up
-        // to 701 tensors, best fit: 39.7 us with 128 threads, 31.1 with 512)
-        int sms = 0;
-        const cudaError_t e = sm_count(&sms);
-        if (e != cudaSuccess) return e;
-        if (g.narrow && g.smem && bt.max_tensors > kFewTensors && bt.n_traces <= 2 * sms)
-            return launch_variant<int16_t, W, true, kFused, kPlanThreadsFew, kTierNone>(bt, g, pw, out, ws, stream);
         // Large components without long-lived members come with many tensors a
         // step: with lifetimes of two steps on average, half a tensor a step makes
         // components of one or two, two a step components of fifteen on average
         // and a hundred at most.  The kernel that can walk them is a little slower
         // for traces without any (4,096 traces of 512 tensors over 1,024 steps:
-        // 108.9 us, 107.0 without the walk).
-        if (g.narrow && g.smem && 4 * (int64_t)bt.max_tensors < 3 * (int64_t)bt.max_steps)
+        // 109.8 us, 106.7 without the walk).
+        const bool crowded = 4 * (int64_t)bt.max_tensors >= 3 * (int64_t)bt.max_steps;
+        // Traces of some length, too few to fill the GPU with 128 threads each:
+        // the latency of one CTA is what counts, and more threads shorten all
+        // but the placement of its longest component (301 ragged traces of up
+        // to 701 tensors, best fit: 39.7 us with 128 threads, 31.1 with 512).
+        // What it leaves to the second launch is better walked where that has no
+        // phases and is more than a wave (160 traces of 4,500 tensors over 2,250
+        // steps: 1.29 ms and 0.69 walked; 40 chains of 4,667, some of whose
+        // components are too large for the walk: 1.69 and 2.19 ms).
+        if (g.narrow && g.smem && bt.max_tensors > kFewTensors &&
+            bt.n_traces <= (phased || !crowded ? 2 * sms : sms))
+            return launch_variant<int16_t, W, true, kFused, kPlanThreadsFew, kTierNone>(bt, g, pw, out, ws, stream);
+        if (g.narrow && g.smem && !crowded)
             return launch_variant<int16_t, W, true, kFused, kSmemThreads, kTierNone>(bt, g, pw, out, ws, stream);
+    } else if (phased) {
+        return g.smem
+                   ? launch_variant<int16_t, W, true, kFused, kSmemThreads, kTierPhases>(bt, g, pw, out, ws, stream)
+                   : launch_variant<int16_t, W, false, kFused, kGlobalThreads, kTierPhases>(bt, g, pw, out, ws, stream);
     }
     constexpr Tier kSmemTier = sizeof(W) == 8 ? kTierCta : kTierWalk;
     constexpr Tier kGlobalTier = sizeof(W) == 8 ? kTierCta : kTierNone;

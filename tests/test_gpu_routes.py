@@ -110,6 +110,21 @@ def test_phases_limits(routes, traces, n, T, route):
     _check(ts)
 
 
+@pytest.mark.parametrize("traces,T,route", ((160, 5466, "walk"), (160, 5467, "general"), (33, 5466, "general")))
+def test_long_traces_without_phases(routes, traces, T, route):
+    """Traces past the phases' limits, and too long on average for a launch that
+    takes the others: walked by 128 threads in a larger batch, with few tensors a
+    step or few traces left to the general path."""
+    rng = np.random.default_rng(T)
+    ts = [_linked(rng, 1020) for _ in range(traces - 1)]
+    _, a, f, s = _trace(rng, 4100, 5000, 0.0, 64, 1 << 14, life=2)
+    ts.append((T, a, f, s))
+    ts = tg.from_arrays(ts)
+    size, _, _ = _plans(ts, routes)
+    assert size == {"first": 1, route: traces - 1}
+    _check(ts)
+
+
 @pytest.mark.parametrize("traces", (40, 160))
 def test_a_long_trace_among_ordinary_ones(routes, traces):
     """One trace past the phases' limits leaves them to the others."""
