@@ -941,11 +941,11 @@ cudaError_t launch_rest(const mp_batch& bt, int32_t policy, int64_t* offsets, in
     if (e == cudaSuccess)
         e = max_resident_ctas((const void*)k_breadth_tensor<kSmem>, kBreadthThreads, smem, &resident);
     if (e != cudaSuccess) return e;
-    // (two waves of CTAs, so that the second evens the first out: a whole CTA for every
-    // trace that has nothing to do costs 1.5 us with 4,096 of them)
-    return launch_next(k_breadth_tensor<kSmem>, (int)std::min<int64_t>(bt.n_traces, 2 * (int64_t)resident),
-                       kBreadthThreads, smem, stream, deferred_only && kSmem, bt, policy, offsets, plan_peak, status,
-                       ws, data, deferred_only);
+    // (two waves of CTAs in a larger batch, so that the second evens the first out: a
+    // whole CTA for every trace costs 1.5 us where 4,096 of them have nothing to do)
+    const int64_t grid = std::min<int64_t>(bt.n_traces, bt.n_traces > 2 * sms ? 2 * (int64_t)resident : resident);
+    return launch_next(k_breadth_tensor<kSmem>, (int)grid, kBreadthThreads, smem, stream,
+                       deferred_only && kSmem, bt, policy, offsets, plan_peak, status, ws, data, deferred_only);
 }
 
 }  // namespace

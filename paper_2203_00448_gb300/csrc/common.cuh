@@ -335,10 +335,10 @@ __device__ int64_t block_incl_scan_max_i64(int64_t* x, int64_t len, int64_t init
 // consecutive bytes; stored straight from registers, 16 bytes every 64, each
 // store touches four times as many cache lines (live profiles of 4,096 traces of
 // 1,024 steps: 20.5 us so, 18.4 this way).
-template <typename W, typename At>
+template <typename W, bool kShort = false, typename At>
 __device__ __forceinline__ void warp_store_profile(int64_t* __restrict__ out, int32_t base, int32_t T, bool vec,
                                                    const W (&v)[8], At&& at) {
-    if (base >= T) return;  // (the whole warp)
+    if (kShort && base >= T) return;  // (the whole warp)
     const int32_t lane = (int32_t)(threadIdx.x & 31), my = base + 8 * lane;
     if (my + 8 <= T) {
         W* run = at(my);  // 16-byte aligned, the 8 words consecutive
@@ -358,7 +358,7 @@ __device__ __forceinline__ void warp_store_profile(int64_t* __restrict__ out, in
     __syncwarp();
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
-        if (base + 64 * r >= T) break;
+        if (kShort && base + 64 * r >= T) break;
         const int32_t t = base + 64 * r + 2 * lane;
         if (t + 1 < T && vec) {
             const W* p = at(t);

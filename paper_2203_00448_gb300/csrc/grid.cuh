@@ -74,20 +74,21 @@ __host__ __device__ inline int64_t chain_room(int64_t n, int64_t nlong, int64_t 
     if (FarLayout((int32_t)n, (int32_t)nlong).total > kFarSmem) return -1;
     if (n <= 1024) return INT32_MAX;
     if (nlong == 0) return -1;
+    // (in floating point: a thread of k_grid_prep does it with everybody waiting)
     const bool first = policy == MP_FIT_FIRST;
-    const int64_t most = 27 * long_steps / (10 * T), hops = most < nlong ? most : nlong;
-    const int64_t seen = n * long_steps / (T * nlong);  // tensors allocated during a long-lived one's life
-    int64_t flow = hops * (1950 + seen) / 130;
-    if (!first) flow = flow * 115 / 100;
-    if (seen > kFlowPairs) flow *= first ? 2 : 4;
-    int64_t phased = 150 + n * n / 120000;
-    if (first) phased += nlong * (5000 + n / 5) / 1000;
-    else phased += (nlong * (7000 + n * 2 / 3) + (nlong - long_steps / T) * (3000 + n * 10 / 9)) / 1000;
-    if (phased > flow) return -1;
-    const int64_t live = 10 * short_steps / T;  // tenths
-    const int64_t member = first ? 930 + (live > 90 ? 11 * (live - 90) : 0) : 400 + 29 * live;  // ns
-    const int64_t room = (flow - phased) * 1000 / member;
-    return room < kLeastRoom ? -1 : room;
+    const float nf = (float)n, longs = (float)nlong, live_long = (float)long_steps / (float)T;
+    const float hops = fminf(2.7f * live_long, longs);
+    const float seen = nf * live_long / longs;  // tensors allocated during a long-lived one's life
+    float flow = hops * (15.0f + seen * (1.0f / 130.0f));
+    if (!first) flow *= 1.15f;
+    if (seen > (float)kFlowPairs) flow *= first ? 2.0f : 4.0f;
+    float phased = 150.0f + nf * nf * (1.0f / 120000.0f);
+    if (first) phased += longs * (5.0f + nf * (1.0f / 5000.0f));
+    else phased += longs * (7.0f + nf * (1.0f / 1500.0f)) + (longs - live_long) * (3.0f + nf * (1.0f / 900.0f));
+    const float live = (float)short_steps / (float)T;
+    const float member = first ? 0.93f + 0.11f * fmaxf(live - 9.0f, 0.0f) : 0.4f + 0.29f * live;
+    const float room = (flow - phased) / member;
+    return room < (float)kLeastRoom ? -1 : (int64_t)room;
 }
 
 // Queues and counters shared by the whole grid.

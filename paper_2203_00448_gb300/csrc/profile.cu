@@ -99,7 +99,7 @@ __device__ __forceinline__ int64_t scan_and_write(W* D, int64_t* out, int32_t T,
         }
         if constexpr (kSmem) {
             // (a warp only rewrites words that it alone has read)
-            warp_store_profile<W>(out, base + (tid & ~31) * kProfItems, T, vec_out, v,
+            warp_store_profile<W, true>(out, base + (tid & ~31) * kProfItems, T, vec_out, v,
                                   [&](int32_t t) { return D + dpos<kSmem, W>(t); });
         } else if (vec_out && my + kProfItems <= T) {
 #pragma unroll
