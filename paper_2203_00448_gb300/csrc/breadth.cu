@@ -775,8 +775,8 @@ k_breadth_comp(mp_batch bt, int32_t policy, int64_t* __restrict__ offsets, int64
 
 // The traces k_breadth_comp deferred (or, with deferred_only false, all of
 // them), in phases where they fit that path (phase_smem: the shared memory for
-// it; 0: none does), else tensor by tensor (by_tensor; otherwise they are left deferred).  It waits for
-// the kernel before it in the kernel.
+// it; 0: none does), else tensor by tensor (by_tensor; otherwise they are left
+// deferred).  It waits for the kernel before it in the kernel.
 template <bool kSmem>
 __global__ void __launch_bounds__(kBreadthPhaseThreads, 1)
 k_breadth_rest(mp_batch bt, int32_t policy, int64_t* __restrict__ offsets, int64_t* __restrict__ plan_peak,
@@ -908,7 +908,7 @@ cudaError_t launch_next(void (*kernel)(Params...), int grid, int threads, size_t
 // and a trace of 5,000 tensors: 15.6 ms in one launch, 5.7 apart).  A batch
 // that is more than one wave of its CTAs is placed tensor by tensor with small ones
 // (1,000 traces of 1,500 tensors, none of them for the phases: 22.7 ms with the
-// phases' registers, 17.1 so).
+// phases' registers, 18.2 so).
 template <bool kSmem>
 cudaError_t launch_rest(const mp_batch& bt, int32_t policy, int64_t* offsets, int64_t* plan_peak, int32_t* status,
                         void* workspace, bool comp, size_t phase_smem, int sms, cudaStream_t stream) {

@@ -56,7 +56,7 @@ constexpr int32_t kTeams = 4;          // ... up to this many of a run
 #ifdef MP_TEST_SPIN_CYCLES
 constexpr int32_t kTeamPolls = 1 << 17;  // test builds: some 6 ms
 #else
-constexpr int32_t kTeamPolls = 1 << 20;  // polls of a wait there (some 50 ms) in which some member has to be placed
+constexpr int32_t kTeamPolls = 1 << 23;  // polls of a wait there (some 0.2 s) in which some member has to be placed
 #endif
 constexpr int32_t kListRun = 64;       // runs from this length on list the gaps between the long tensors first
 constexpr int32_t kFewPending = 8;     // up to this many are inserted by comparison with every entry
@@ -147,8 +147,9 @@ template <bool kBreadth>
 size_t smem_bytes(const mp_batch& bt, int sms) {
     if (fits<kBreadth>(bt.max_tensors, bt.max_steps, kSmemCeiling))
         return Layout(bt.max_tensors, bt.max_steps, step_bytes<kBreadth>()).total;
-    if (bt.n_tensors / bt.n_traces > kMixedTensors) return 0;
-    return bt.n_traces > sms ? kTwoPerSm : kSmemCeiling;
+    const size_t room = bt.n_traces > sms ? kTwoPerSm : kSmemCeiling;
+    const int64_t n = bt.n_tensors / bt.n_traces, T = bt.n_steps / bt.n_traces;  // of the average trace
+    return n <= kMixedTensors && T <= 65535 && fits<kBreadth>((int32_t)n, (int32_t)T, room) ? room : 0;
 }
 
 struct Shared {
@@ -157,7 +158,7 @@ struct Shared {
     uint32_t best32, lb, far;
     int32_t bad, lw, nl, cnt, next, cnt1, next1, teams, fail;
     int32_t seen[16];  // by warp: members of its team placed when it last asked
-    int32_t hold;    // test builds: alloc-order position of a team's member that is never placed (-1: none)
+    int32_t hold;      // test builds: alloc-order position of a team's member that is never placed (-1: none)
     uint16_t team[kTeams];
     uint32_t last_free;
     uint32_t before[kFewPending];
@@ -1340,8 +1341,8 @@ static __device__ __noinline__ void sort_keys(int32_t n) {
 // with nothing written, when the trace is not one for this path: an invalid
 // tensor, sizes summing to 2^32 units or more, too many long tensors, or a long
 // chain beside some.  That is known before the sorts, so that a trace for the
-// general path loses little here (REFUSEDUS), and no thread touches the dynamic
-// shared memory any more when another one returns.
+// general path loses little here, and no thread touches the dynamic shared memory
+// any more when another one returns.
 template <bool kBreadth, bool kCheck>
 __device__ __forceinline__ bool plan(const mp_batch& bt, const TraceView& tv, int32_t policy, const Out& out) {
     extern __shared__ __align__(16) unsigned char smem_raw[];

@@ -2293,7 +2293,8 @@ cudaError_t launch_width(const mp_batch& bt, const PlanOut& out, unsigned char* 
         // and a hundred at most.  The kernel that can walk them is a little slower
         // for traces without any (4,096 traces of 512 tensors over 1,024 steps:
         // 109.8 us, 106.7 without the walk).
-        const bool crowded = 4 * (int64_t)bt.max_tensors >= 3 * (int64_t)bt.max_steps;
+        const bool crowded =
+            bt.max_tensors > kWarpComp && 4 * (int64_t)bt.max_tensors >= 3 * (int64_t)bt.max_steps;
         // Traces of some length, too few to fill the GPU with 128 threads each:
         // the latency of one CTA is what counts, and more threads shorten all
         // but the placement of its longest component (301 ragged traces of up
