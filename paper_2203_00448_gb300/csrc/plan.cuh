@@ -101,7 +101,9 @@ constexpr int32_t kSpinPolls = 64;   // polls of a queue slot before the waiting
 constexpr int32_t kDeferred = -1;    // trace status between the two launches: left to the second
 constexpr int32_t kWalkComp = 1024;  // the walk tier's largest component
 constexpr int32_t kWalkFew = 128;    // ... where the second launch holds the whole batch at once
-constexpr int32_t kWalkWindow = 128; // ... and where it does not, the average window of a component
+constexpr int32_t kWalkWindow = 135; // ... and where it does not, the average window of a component
+constexpr int32_t kWalkWork = 41000; // ... and the sum of its windows, the more the more traces (walk_rule)
+constexpr int32_t kWalkHeld = 128;   // window positions a warp holds in registers
 constexpr int32_t kWalkComps = 64;   // components a trace may have there
 constexpr int kLifeBits = 6;         // bits of a short-lived tensor's life (at most kLongLife)
 
@@ -1436,9 +1438,10 @@ __device__ __forceinline__ W large_tier(const ARec<I, W>* AR, W* OFFP, const int
 
 // Which large components the first launch walks: those of at most `comp`
 // members, none of them long-lived, whose windows (the alloc-order positions
-// that can overlap a member) have `window` positions on average or fewer.
+// that can overlap a member) have at most `window` positions on average and `work`
+// in all.
 struct WalkRule {
-    int32_t comp, window;
+    int32_t comp, window, work;
 };
 
 // Looks the nx large components starting at LST[0, nx) over, a warp each, and
@@ -1464,7 +1467,8 @@ __device__ __forceinline__ bool walk_refuses(const ARec<I, W>* AR, const int32_t
             const int32_t a = AR[p0 + k].a, f = AR[p0 + k].f;
             sum += min(p0 + c, BEND[f - 1]) - max(p0, a >= lw ? BEND[a - lw] : 0);
         }
-        if (__reduce_add_sync(full, sum) / c > rule.window) return true;
+        sum = __reduce_add_sync(full, sum);
+        if (sum > rule.work || sum / c > rule.window) return true;
         if (lane == 0) large[qc] = (p0 << kLifeBits) | lw;
     }
     return false;
@@ -1577,7 +1581,7 @@ __device__ __forceinline__ W walk_tier(ARec<I, W>* AR, W* OFFP, const int32_t* B
                 });
             } else {
                 // a window too wide for a mask: the predecessors at its first
-                // kWalkWindow positions are held as above, those past them found on
+                // kWalkHeld positions are held as above, those past them found on
                 // every pass (2,048 traces of 512 tensors over 100 steps: 1.76 ms
                 // with all of them found on every pass, 0.75 so)
                 const int32_t w0 = -1 - (int32_t)me.pad, w1 = min(p0 + c, BEND[(int32_t)me.f - 1]);
@@ -1589,13 +1593,13 @@ __device__ __forceinline__ W walk_tier(ARec<I, W>* AR, W* OFFP, const int32_t* B
                     po = voff[q];
                     return (W)(po + oq.s);
                 };
-                W co[kWalkWindow / 32], ce[kWalkWindow / 32];
+                W co[kWalkHeld / 32], ce[kWalkHeld / 32];
 #pragma unroll
-                for (int u = 0; u < kWalkWindow / 32; ++u) ce[u] = end_of(w0 + lane + 32 * u, co[u]);
+                for (int u = 0; u < kWalkHeld / 32; ++u) ce[u] = end_of(w0 + lane + 32 * u, co[u]);
                 place([&](auto&& fn) {
 #pragma unroll
-                    for (int u = 0; u < kWalkWindow / 32; ++u) fn(co[u], ce[u]);
-                    for (int32_t q = w0 + kWalkWindow + lane; q < w1; q += 32) {
+                    for (int u = 0; u < kWalkHeld / 32; ++u) fn(co[u], ce[u]);
+                    for (int32_t q = w0 + kWalkHeld + lane; q < w1; q += 32) {
                         W po;
                         const W pe = end_of(q, po);
                         fn(po, pe);
@@ -2160,10 +2164,10 @@ k_plan(mp_batch bt, PlanOut out, unsigned char* __restrict__ ws, size_t data_str
 template <bool kFused>
 __global__ void __launch_bounds__(kPlanThreadsSmem, 4) k_plan_small(mp_batch bt, PlanOut out) {
     const int b = blockIdx.x;
-    plan_trace<int16_t, uint32_t, true, kFused, kTierNone>(b, bt, out, nullptr, 0, 0, 0, {0, 0});
+    plan_trace<int16_t, uint32_t, true, kFused, kTierNone>(b, bt, out, nullptr, 0, 0, 0, {0, 0, 0});
     __syncthreads();
     if (*(volatile int32_t*)(out.status + b) != kDeferred) return;
-    plan_trace<int16_t, int64_t, true, kFused, kTierNone>(b, bt, out, nullptr, 0, 0, 0, {0, 0});
+    plan_trace<int16_t, int64_t, true, kFused, kTierNone>(b, bt, out, nullptr, 0, 0, 0, {0, 0, 0});
 }
 
 struct PlanGeometry {
@@ -2212,19 +2216,22 @@ PlanWorkspace plan_workspace(const mp_batch& bt) {
 // before it has begun (chains of 94: 53 us walked, 78 in phases).  In a larger
 // batch every warp walks: the first launch holds nine traces an SM, the phases two
 // (600 / 4,096 chains of 374: 160 / 553 us walked, 234 / 1,395 in phases; 4,096
-// traces of 1,000 random tensors over 400 steps 1.02 and 1.72 ms), up to the
-// windows a warp holds in registers (walk_tier); past them every level of a stack
-// is another look through the window (1,024 traces of 1,000 tensors over 30 steps:
-// 73 ms walked, 30 in phases).
+// traces of 1,000 random tensors over 400 steps 1.02 and 1.72 ms).  Past the
+// windows a warp holds in registers every level of a stack is another look through
+// the window (1,024 traces of 1,000 tensors over 30 steps: 73 ms walked, 30 in
+// phases), and the second launch waits for the slowest walk: what is walked in a
+// batch of some of either kind has to be little beside what is left, hence the
+// bound on the work (600 traces of 600 tensors over 60 steps, some of whose windows
+// are narrow enough: 3.78 ms without it, 2.40 with none walked).
 template <bool kFused>
 WalkRule walk_rule(const mp_batch& bt, int sms) {
     const PlanGeometry wide = plan_geometry<int64_t>(bt, kFused);
     const size_t phase_smem = wide.narrow ? phases::smem_bytes<false>(bt, sms) : 0;
-    if (phase_smem == 0) return {kWalkComp, kWalkComp};
+    if (phase_smem == 0) return {kWalkComp, kWalkComp, INT32_MAX};
     const size_t smem = std::max(wide.smem ? wide.data : flow_smem_bytes<int64_t>(), phase_smem);
     if (bt.n_traces <= (smem <= kTwoPerSm ? 2 * sms : sms))
-        return {bt.max_tensors <= kWalkFew ? kWalkFew : kWarpComp, kWalkComp};
-    return {kWalkComp, kWalkWindow};
+        return {bt.max_tensors <= kWalkFew ? kWalkFew : kWarpComp, kWalkComp, INT32_MAX};
+    return {kWalkComp, kWalkWindow, kWalkWork * std::clamp(bt.n_traces / (6 * sms), 1, 32)};
 }
 
 template <typename I, typename W, bool kSmem, bool kFused, int kThreads, Tier kTier>
@@ -2242,7 +2249,7 @@ cudaError_t launch_variant(const mp_batch& bt, const PlanGeometry& g, const Plan
     smem = std::max(smem, phase_smem);
     // more traces than SMs: half the threads, where an SM holds two of them
     if (phase_smem > 0 && bt.n_traces > sms && smem <= kTwoPerSm) threads /= 2;
-    const WalkRule rule = kTier == kTierWalk ? walk_rule<kFused>(bt, sms) : WalkRule{0, 0};
+    const WalkRule rule = kTier == kTierWalk ? walk_rule<kFused>(bt, sms) : WalkRule{0, 0, 0};
     const void* fn = (const void*)k_plan<I, W, kSmem, kFused, kThreads, kTier>;
     {
         cudaError_t e = set_smem_limit(fn, smem);

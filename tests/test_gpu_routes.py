@@ -48,19 +48,22 @@ def test_chains(routes, traces, n, route):
     _check(ts)
 
 
-# a step's tensors: windows of 2.8 times as many positions on average, on either side of the rule's line
-@pytest.mark.parametrize("traces,per_step,route", ((34, 16, "phases"), (310, 46, "walk"), (310, 47, "phases"),
-                                                   (1000, 46, "walk")))
-def test_wide_windows(routes, traces, per_step, route):
+# a step's tensors: windows of 2.8 times as many positions on average, on either side of the rule's lines for the
+# average (48 a step: 134 positions) and the sum (38 a step: 106, 40,432 for 380 members; twice that with 1,824 traces)
+@pytest.mark.parametrize("traces,steps,per_step,route", ((34, 10, 16, "phases"), (310, 10, 38, "walk"), (310, 10, 39, "phases"),
+                                                         (310, 5, 52, "walk"), (310, 5, 53, "phases"),
+                                                         (1824, 10, 48, "walk"), (1824, 10, 49, "phases"),
+                                                         (1823, 10, 48, "phases")))
+def test_wide_windows(routes, traces, steps, per_step, route):
     rng = np.random.default_rng(per_step + traces)
     ts = []
     for k in range(traces):
-        if k % 50:
+        if k % 100:
             ts.append(_small(rng))
             continue
-        a = np.repeat(np.arange(10), per_step)  # each lives two steps
-        ts.append((12, a, a + 2, rng.integers(1, 1 << 10, len(a)) * 64))
-    big = (traces + 49) // 50
+        a = np.repeat(np.arange(steps), per_step)  # each lives two steps
+        ts.append((steps + 2, a, a + 2, rng.integers(1, 1 << 10, len(a)) * 64))
+    big = (traces + 99) // 100
     ts = tg.from_arrays(ts)
     size, _, _ = _plans(ts, routes)
     assert size == {"first": traces - big, route: big}
