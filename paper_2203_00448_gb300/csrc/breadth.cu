@@ -900,6 +900,10 @@ cudaError_t launch_next(void (*kernel)(Params...), int grid, int threads, size_t
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+constexpr int32_t kBApart = 1024;  // launch_rest
+// Enough tensors a step for dense traces, as comp_rule has them.
+bool crowded(const mp_batch& bt) { return 4 * (int64_t)bt.max_tensors >= 3 * (int64_t)bt.max_steps; }
+
 // What k_breadth_comp leaves (comp; otherwise all traces).  Both ways in one launch
 // where that holds the batch at once and what places tensor by tensor wants no
 // shared memory that the phases do not leave it -- 256 traces of 2,000 tensors take
@@ -908,7 +912,8 @@ cudaError_t launch_next(void (*kernel)(Params...), int grid, int threads, size_t
 // and a trace of 5,000 tensors: 15.6 ms in one launch, 5.7 apart).  A batch
 // that is more than one wave of its CTAs is placed tensor by tensor with small ones
 // (1,000 traces of 1,500 tensors, none of them for the phases: 22.7 ms with the
-// phases' registers, 18.2 so).
+// phases' registers, 18.2 so) where that may be for many of its traces or matters
+// more than a launch: 1.6 us, 8% of the call for 500 traces of 60 tensors.
 template <bool kSmem>
 cudaError_t launch_rest(const mp_batch& bt, int32_t policy, int64_t* offsets, int64_t* plan_peak, int32_t* status,
                         void* workspace, bool comp, size_t phase_smem, int sms, cudaStream_t stream) {
@@ -927,7 +932,8 @@ cudaError_t launch_rest(const mp_batch& bt, int32_t policy, int64_t* offsets, in
     cudaError_t e = rest_geometry<kSmem>(bt, phase_smem, true, sms, &g);
     if (e != cudaSuccess) return e;
     if (phase_smem > 0) {
-        if (bt.n_traces <= g.resident && kSmem && data <= std::max(phase_smem, kTwoPerSm)) return rest(phase_smem, true);
+        const bool small_ctas = bt.n_traces > g.resident && (bt.max_tensors > kBApart || crowded(bt));
+        if (!small_ctas && kSmem && data <= std::max(phase_smem, kTwoPerSm)) return rest(phase_smem, true);
         e = rest_geometry<kSmem>(bt, phase_smem, false, sms, &g);
         if (e == cudaSuccess) e = rest(phase_smem, false);
         deferred_only = true;

@@ -203,15 +203,17 @@ def test_breadth_dense(routes, traces, per_step, route):
     _check(ts)
 
 
-def test_breadth_tensor_by_tensor_with_small_ctas(routes):
-    """More traces than the phases' launch holds at once, some of which it refuses."""
+@pytest.mark.parametrize("T", (400, 401))
+def test_breadth_tensor_by_tensor_in_large_batches(routes, T):
+    """More traces than the phases' launch holds at once, some of which it refuses:
+    by a launch of their own with many tensors a step, else by the phases' launch."""
     rng = np.random.default_rng(3)
     ts = [_small(rng) for _ in range(400)]
     for k in (0, 199, 399):
-        T, a, f, s = _trace(rng, 300, 400, 0.05, 1, 1 << 10, full_span=True)
+        _, a, f, s = _trace(rng, 300, 400, 0.05, 1, 1 << 10, full_span=True)
         s[0] = (1 << 40) + 1
         ts[k] = (T, a, f, s)
-    ts[7] = _trace(rng, 300, 400, 0.05, 1, 1 << 10, full_span=True)
+    ts[7] = _trace(rng, 300, T, 0.05, 1, 1 << 10, full_span=True)
     ts = tg.from_arrays(ts)
     got = _plans(ts, routes)[1:]
     assert got[0] == got[1] == {"breadth-comp": 396, "breadth-phases": 1, "breadth-tensor": 3}
